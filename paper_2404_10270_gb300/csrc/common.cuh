@@ -102,14 +102,14 @@ struct SegParams {
     int32_t pad;
 };
 
-// A segment whose fixed-point deposit is kept from step to step instead of being formed
-// anew: a neutral particle target that moves only on some steps (subcycled).  Its
-// charge is 0, so the kept deposit serves the density diagnostic alone; the mover
-// skips its tiles between its moves and, on a move, takes the old positions' share
-// away and adds the new one; a conversion into an ion takes the particle's share away.
-__host__ __device__ __forceinline__ bool deposit_kept(const SegParams& P)
+// Whether a species with subcycling moves on step n (counted from 0).  On the steps it
+// rests its fixed-point deposit stands: the field phase before such a step does not clear
+// it, the mover leaves the segment's tiles alone, and what the event kernels create or
+// convert is added or taken away as on every step (integer sums, so the standing deposit
+// equals a fresh one bit for bit).
+__host__ __device__ __forceinline__ bool moves_on(const SegParams& P, int64_t n)
 {
-    return P.is_target != 0 && P.nstep > 1;
+    return P.nstep == 1 || (n + 1) % P.nstep == 0;
 }
 
 // The origin of a segment's clocks at step n (loads and reads count from it): its own

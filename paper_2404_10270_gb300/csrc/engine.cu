@@ -586,11 +586,6 @@ int launch_move(pic_handle* h, bool move, int phase = kPlain)
         const bool pair = move && !sort && !h->any_mag && h->precision == PIC_FP32 &&
                           h->total_cap >= h->pair_min && h->pair_ok;
         a.pair = pair ? 1 : 0;
-        // the step on which the neutral particle targets move (they all have the sort
-        // interval as their subcycling factor): the variant that updates their kept
-        // deposit; on the other steps their tiles are skipped
-        const bool kept = move && h->any_target && h->sort_interval > 1 &&
-                          (h->step_h + 1) % h->sort_interval == 0;
         for (int v = 0; v < (pair ? 2 : 1); ++v) {
             h->kernels += 1;
             const bool lean = v == 1;
@@ -598,10 +593,10 @@ int launch_move(pic_handle* h, bool move, int phase = kPlain)
             const bool gridv = pair && !lean && !h->any_subcycle;
             const cudaError_t e =
                 h->precision == PIC_FP64
-                    ? launch_move_f64(a, mag, move, h->any_subcycle, h->any_unmag, sort, kept,
+                    ? launch_move_f64(a, mag, move, h->any_subcycle, h->any_unmag, sort,
                                       sort ? h->nt_sort : h->nt, grid, h->stream)
                     : launch_move_f32(a, mag, move, h->any_subcycle, h->any_unmag, sort, lean,
-                                      gridv, kept, sort ? h->nt_sort : h->nt,
+                                      gridv, sort ? h->nt_sort : h->nt,
                                       gridv ? h->grid_test : grid, h->stream);
             CUDA_TRY(h, e);
         }
@@ -677,7 +672,7 @@ int ensure_fields(pic_handle* h)
     if (h->any_target && (rc = do_sort(h))) return rc;
     rc = launch_tiles_h(h);
     if (rc) return rc;
-    // a fresh deposit of every particle (kept deposits start over too)
+    // a fresh deposit of every particle (those that stand start over too)
     CUDA_TRY(h, cudaMemsetAsync(h->dep, 0, sizeof(unsigned long long) * (size_t)h->seg_nodes, h->stream));
     if ((rc = launch_move(h, false))) return rc;
     {
@@ -1851,6 +1846,8 @@ int pic_restore_counters(pic_handle* h, int64_t step, const uint64_t* next_id)
         CUDA_TRY(h, cudaMemcpy(h->next_id, next_id, 8 * (size_t)h->ninst, cudaMemcpyHostToDevice));
     }
     CUDA_TRY(h, cudaMemset(h->test_all, 1, sizeof(int)));
+    // which deposits stand depends on the step a subcycled species next moves on
+    if (step != h->step_h && h->any_subcycle) h->stale = true;
     h->step_h = step;
     h->hist_ready = false;
     return PIC_OK;

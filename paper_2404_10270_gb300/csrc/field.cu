@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(kChunkThreads) k_field_emit(const FieldArgs f,
     const int b = f.chunk_inst[c];
     const InstParams& I = f.inst[b];
     const int N = I.ncells;
+    const int64_t next = f.step[0] + (advance ? 1 : 0);
     const int a = (c - I.chunk0) * kChunk;
     const int j0 = a + threadIdx.x * kChunkPer;
     const bool poisson = I.field == PIC_FIELD_POISSON;
@@ -190,12 +191,12 @@ __global__ void __launch_bounds__(kChunkThreads) k_field_emit(const FieldArgs f,
         z[t] = 0;
         if (j > N) continue;
         // the deposit hand-over: keep the last complete deposit, clear for the next step
-        // (a kept deposit, deposit_kept(), is updated in place instead)
+        // (that of a species which rests on the next step stands, moves_on())
         for (int k = 0; k < I.nseg; ++k) {
             const SegParams& P = f.seg[I.seg0 + k];
             const unsigned long long d = f.dep[P.node + j];
             f.dep_last[P.node + j] = d;
-            if (!deposit_kept(P)) f.dep[P.node + j] = 0ull;
+            if (moves_on(P, next)) f.dep[P.node + j] = 0ull;
             z[t] += (i128)I.z[k] * (i128)(long long)d;
         }
         if (I.smooth && poisson) z[t] = f.zs[I.inode + j];

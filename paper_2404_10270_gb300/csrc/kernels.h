@@ -17,14 +17,12 @@ struct MoveArgs;
 // without magnetic field): the variant that queues collision-clock tests for the event
 // kernel instead of drawing them inline; `gridv`: the inline-test partner of the mover
 // pair, which runs only on the steps where every clock tests (without subcycling: the
-// variant that draws a quad's four tests side by side); `kept`: the neutral particle
-// targets (whose deposit is kept from step to step) move on this step (on the other
-// steps their tiles are skipped).  Returns the launch error.
+// variant that draws a quad's four tests side by side).  Returns the launch error.
 cudaError_t launch_move_f32(const MoveArgs& a, bool mag, bool move, bool sub, bool mixed,
-                            bool sort, bool lean, bool gridv, bool kept, int nt, int grid,
+                            bool sort, bool lean, bool gridv, int nt, int grid,
                             cudaStream_t st);
 cudaError_t launch_move_f64(const MoveArgs& a, bool mag, bool move, bool sub, bool mixed,
-                            bool sort, bool kept, int nt, int grid, cudaStream_t st);
+                            bool sort, int nt, int grid, cudaStream_t st);
 // The rare events the mover queued this step (events.cu): collision candidates, clock
 // tests and wall hits, one thread each, `grid` blocks of 128 threads.
 cudaError_t launch_events(const MoveArgs& a, int precision, int grid, cudaStream_t st);

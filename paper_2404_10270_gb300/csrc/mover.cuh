@@ -301,8 +301,7 @@ __device__ __forceinline__ void st4(double* p, const double v[4])
 // goes to HBM on its own.
 // jd = -1 marks an empty slot: as unsigned it is never the minimum of a live cell, as
 // signed never the maximum, and it matches no cell.
-// NEG: take the quad's charge away instead (two's complement sums; the counts are not
-// touched), for a particle deposit that is kept from step to step and updated.
+// gdep null (OPT variants): only the counts, for a species whose deposit stands.
 constexpr int kDepLoopCells = 6;  // register reductions up to this many cells
 
 // Words of a warp's deposit window: 32 counts and 32 charge sums (FP64: the 48-bit
@@ -322,7 +321,7 @@ __device__ __forceinline__ void dep_win_clear(uint32_t* win)
     __syncwarp();
 }
 
-template <typename Q, bool NEG = false>
+template <typename Q, bool OPT = false>
 __device__ __forceinline__ void warp_deposit(const int jd[4], const Q qr[4],
                                              unsigned long long S,
                                              unsigned long long* __restrict__ gdep,
@@ -425,10 +424,10 @@ __device__ __forceinline__ void warp_deposit(const int jd[4], const Q qr[4],
             __syncwarp();
         }
         const unsigned long long prevR = __shfl_up_sync(FULL, myR, 1);
-        if (lane <= ncell) {
+        if (lane <= ncell && (!OPT || gdep)) {
             const unsigned long long tot =
                 S * (unsigned long long)myn - myR + (lane > 0 ? prevR : 0ull);
-            if (tot != 0) atomicAdd(gdep + wmin + lane, NEG ? 0ull - tot : tot);
+            if (tot != 0) atomicAdd(gdep + wmin + lane, tot);
         }
         // the particles per cell, for a sort in the next step
         if (ghist && lane < ncell && myn != 0u) atomicAdd(ghist + wmin + lane, myn);
@@ -437,8 +436,10 @@ __device__ __forceinline__ void warp_deposit(const int jd[4], const Q qr[4],
         for (int k = 0; k < 4; ++k)
             if (jd[k] >= 0) {
                 const unsigned long long l = S - (unsigned long long)qr[k], r = qr[k];
-                atomicAdd(gdep + jd[k], NEG ? 0ull - l : l);
-                atomicAdd(gdep + jd[k] + 1, NEG ? 0ull - r : r);
+                if (!OPT || gdep) {
+                    atomicAdd(gdep + jd[k], l);
+                    atomicAdd(gdep + jd[k] + 1, r);
+                }
                 if (ghist) atomicAdd(ghist + jd[k], 1u);
             }
     }
@@ -645,13 +646,13 @@ __device__ __forceinline__ void queue_rare(const MoveArgs& a, int s, unsigned ca
 // magnetized and unmagnetized instances, so the push is chosen per segment.
 // TEST: the collision-clock test (a Philox draw and a table search) runs inline;
 // without it a particle whose clock needs a test is queued for the event kernel, which
-// keeps the common path free of the draw's code and registers.  KEPT: the step on which
-// the neutral particle targets (whose deposit is kept, deposit_kept()) move; on every
-// other step their tiles are skipped (a separate variant, so that the update's
-// registers do not burden the common steps).  (The step that ends a sort cycle runs
-// k_move_sort below instead.)
+// keeps the common path free of the draw's code and registers.  A segment that rests on
+// this step (subcycling, a neutral particle target) keeps its deposit, so its tiles are
+// skipped, or only counted per cell on the step before a sort: the 30,011-cell plasma
+// with ions moved every fourth step (42 M particles, FP32) went from 212 to 183 us a step.  (The step that
+// ends a sort cycle runs k_move_sort below instead.)
 template <typename T, int NT, bool MAG, bool MOVE, bool SUB, bool MIXED, bool TEST,
-          bool KEPT = false, bool GRID = false>
+          bool GRID = false>
 __global__ void __launch_bounds__(NT, MoveOccupancy<T, MAG, NT, MOVE && SUB && TEST, GRID>::blocks)
 k_move(const __grid_constant__ MoveArgs a)
 {
@@ -699,11 +700,9 @@ k_move(const __grid_constant__ MoveArgs a)
                 moves = ks == 1 || q * ks == step + 1;
                 dgrid = kGapMax - (int)((q - 1) % kGapMax);
                 mown = q - 1;
-                // a neutral particle target keeps its deposit from step to step (the
-                // field phase does not clear it; conversions into ions take their share
-                // away): between its moves nothing of it changes, so the warp goes on
-                // with its first tile past the segment
-                if (!moves && deposit_kept(a.seg[s])) {
+                // a species that rests keeps its deposit: the warp goes on with its first
+                // tile past the segment
+                if (!moves && !a.hist_out) {
                     tile += ((s_end - 1 - tile) / wstride) * wstride;
                     continue;
                 }
@@ -745,19 +744,6 @@ k_move(const __grid_constant__ MoveArgs a)
 #pragma unroll
             for (int k = 0; k < 4; ++k) gq[k] = gap_steps(P.gap, P.glog, w[k]);
         }
-        if (KEPT && MOVE && SUB && moves && deposit_kept(P)) {
-            // its move: the old positions' charge leaves the kept deposit (the new
-            // positions' joins it below), exactly as a fresh deposit would come out
-            int jd[4];
-            Q qr[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                jd[k] = (c[k] >> 31) | (int)((uint32_t)c[k] & kCellMask);
-                if (jd[k] >= 0 && !in_range(a.err, jd[k], 0, P.ncells)) jd[k] = -1;
-                qr[k] = c[k] >= 0 ? (Q)Prec<T>::qright(f[k]) : (Q)0;
-            }
-            warp_deposit<Q, true>(jd, qr, Prec<T>::S, a.dep + node0, nullptr, dwin);
-        }
         if (MOVE && (!SUB || moves)) {
             unsigned cand = 0, wlo = 0, whi = 0, tst = 0, chg = 0;
             quad_physics<T, MAG, false, TEST, GRID>(a, P, smag, step, mown, dgrid, slot, idq, c, f,
@@ -788,8 +774,9 @@ k_move(const __grid_constant__ MoveArgs a)
             if (jd[k] >= 0 && !in_range(a.err, jd[k], 0, P.ncells)) jd[k] = -1;
             qr[k] = c[k] >= 0 ? (Q)Prec<T>::qright(f[k]) : (Q)0;
         }
-        warp_deposit<Q>(jd, qr, Prec<T>::S, a.dep + node0,
-                        a.hist_out ? a.hist_out + node0 : nullptr, dwin);
+        warp_deposit<Q, MOVE && SUB>(jd, qr, Prec<T>::S,
+                                     MOVE && SUB && !moves ? nullptr : a.dep + node0,
+                                     a.hist_out ? a.hist_out + node0 : nullptr, dwin);
     }
 }
 
@@ -1061,7 +1048,8 @@ k_move_sort(const __grid_constant__ MoveArgs a)
             }
             queue_rare(a, s, cand, wlo, whi, tst, to);
         }
-        // 6. deposit of the new positions
+        // 6. deposit of the new positions (that of a segment that rests stands)
+        if (SUB && !moves) continue;
         int jd[4];
         Q qr[4];
 #pragma unroll
