@@ -146,13 +146,14 @@ typedef struct {
                                    first steps of the run (results do not depend on either
                                    choice) and caches the choice per GPU and size bucket
                                    in $BITPIC_TUNE_CACHE (default
-                                   $HOME/.cache/bitpic/autotune.json).  An FP32 batch
-                                   without magnetic field, whose colliding species move
-                                   on every step, with at least $BITPIC_PAIR_MIN_SLOTS
-                                   particle slots (default 2^24) moves its particles
-                                   with a mover variant that leaves most collision-clock
-                                   draws to the event kernel; this too changes no
-                                   result. */
+                                   $HOME/.cache/bitpic/autotune.json).  A batch with at
+                                   least $BITPIC_PAIR_MIN_SLOTS particle slots (default
+                                   2^24) has its own mover variant for the steps on which
+                                   every collision clock tests; from $BITPIC_AHEAD_TILES
+                                   (2) tiles of 128 particles per resident warp the mover
+                                   fetches them ahead, and from $BITPIC_CHUNK_ROUNDS (200)
+                                   its warps take several consecutive tiles; this too
+                                   changes no result. */
     const pic_instance* inst;   /* n_instances entries, copied */
     void* cuda_stream;          /* borrowed cudaStream_t; NULL = library-owned stream */
 } pic_config;

@@ -5,7 +5,8 @@
 //   k_tiles     snapshot each segment's slot count (rounded to a whole quad), build the
 //               tile list, empty the rare-event queue
 //   k_move      gather, push, move, periodic wrap, collision clock, fixed-point deposit;
-//               walls and collision candidates are queued (mover.cuh)
+//               walls and collision candidates are queued (mover.cuh); a large batch takes
+//               another variant on the steps on which every clock tests
 //   k_events    the queued walls and candidates: counters, re-injection, kinematics,
 //               creations (events.cuh)
 //   k_victims   neutral particle targets: the ionized targets become ions (events.cuh)
@@ -72,10 +73,12 @@ void set_global_error(const std::string& msg) { g_create_error = msg; }
 struct pic_handle {
     int precision = PIC_FP32;
     int ninst = 0, nseg = 0, sort_interval = 0, nt = 256, grid_move = 0, sms = 0;
+    MoveMode mode = MoveMode::kDirect;  // the mover variant of a plain step
     size_t tsize = 4;
     std::vector<pic_instance> inst;
     std::vector<SegParams> segh;
     std::vector<InstParams> insth;
+    int64_t max_tiles = 0;  // tiles of full segments
     int64_t total_cap = 0, seg_nodes = 0, inst_nodes = 0, max_cap = 0, ev_total = 0;
     int64_t rare_cap = 0;  // entries of the per-step rare-event queue
     int max_nodes = 0;
@@ -119,9 +122,11 @@ struct pic_handle {
     // the first kernel of every step), [1] the steps completed (the field phase of a
     // step writes [0] + 1), so that the field phase may run beside the event kernels
     int64_t* step_d = nullptr;
-    int* test_all = nullptr;  // nonzero: every clock may need a test in the next step (after a load)
-    int64_t pair_min = (int64_t)1 << 24;  // particle slots from which plain FP32 steps use the mover pair
-    bool pair_ok = true;                  // every colliding species moves on every step
+    bool test_all = true;  // every clock may need a test in the next step (after a load)
+    int64_t full_min = (int64_t)1 << 24;  // particle slots from which test steps take the kFull mover
+    int64_t ahead_tiles = 2;    // tiles per resident warp from which the mover fetches them ahead
+    int64_t chunk_rounds = 200; // tiles per resident warp from which its warps take chunks of tiles
+    std::vector<int> collide_nsteps;      // the distinct subcycling factors of colliding species
     double *kin = nullptr, *phi_d = nullptr;
     std::vector<void*> allocs;
     char* io = nullptr;       // staging of pic_load_particles / pic_get_particles host data
@@ -143,7 +148,7 @@ struct pic_handle {
     // the host, and by the sort that used it); grid of the sorting mover
     bool hist_ready = false;
     int grid_sort = 0;
-    int grid_test = 0;  // grid of the mover pair's inline-test partner (FP32, no subcycling)
+    int grid_full = 0;  // grid of the mover's kFull variant
     // threads per block of the step that ends a sort cycle, apart from the other steps':
     // its four block-wide barriers a chunk cost less in small blocks, while the plain
     // mover gains from large ones (196.6 M particles, FP32: the sort step 2.22 / 2.31 /
@@ -450,6 +455,7 @@ MoveArgs move_args(pic_handle* h)
     a.nseg = h->nseg;
     a.tile_start = h->tile_start;
     a.seg_nmove = h->seg_nmove;
+    a.chunk = 1;
     a.seg_n = h->seg_n;
     a.seg_live = h->seg_live;
     a.accel = h->accel;
@@ -476,8 +482,6 @@ MoveArgs move_args(pic_handle* h)
     a.did = nullptr;
     a.yp = S.yp;
     a.dyp = nullptr;
-    a.test_all = h->test_all;
-    a.pair = 0;
     return a;
 }
 
@@ -538,6 +542,33 @@ FieldArgs field_args(pic_handle* h)
     return f;
 }
 
+// Whether the mover of step n takes its kFull variant: the clocks of a whole species may
+// test, after a load (any batch) or when the species' own step is a multiple of kGapMax
+// (large batches).  The other variants handle such a step too, one particle at a time:
+// below some 16 M slots that costs less than it saves to keep the step inside a captured
+// window (1.6 M particles: under 1 % of the time, averaged over 127 steps).
+bool full_step(const pic_handle* h, int64_t n)
+{
+    for (int K : h->collide_nsteps)
+        if ((n + 1) % K == 0 &&
+            ((h->test_all && n == h->step_h) ||
+             (h->total_cap >= h->full_min && ((n + 1) / K - 1) % kGapMax == 0)))
+            return true;
+    return false;
+}
+
+// Large batches: a warp of the mover takes kMoveChunk consecutive tiles (FP64: twice that)
+// and its block ends, instead of walking the store on a grid of resident blocks.  Blocks
+// start in order as others end, so all warps work on one moving window of the store;
+// on the resident grid they drift apart and HBM sees many places at once.  196.6 M
+// particles, FP32, 256-thread blocks: 0.644 ms against 0.692 (16 tiles 0.646, 32 0.664);
+// FP64 1.41 (16 tiles; 8: 1.43) against 1.47; 128 magnetized instances, FP32: 0.938 against
+// 1.060.  Below chunk_rounds tiles per resident warp the resident grid wins, whose warps
+// are set up once (98 M particles, 158 tiles a warp: 389 against 392 us a step; 49 M: 199
+// against 207; 30 M: 131 against 133), and so it does for the FP64 Boris form, which the
+// FP64 pipe bounds.
+constexpr int kMoveChunk = 8;
+
 // Phases of a time step with respect to the sort folded into it.
 enum StepPhase { kPlain = 0, kCount = 1, kSortStep = 2 };
 
@@ -572,34 +603,24 @@ int launch_move(pic_handle* h, bool move, int phase = kPlain)
     }
     {
         Span sp(h, sort ? 5 : 0);
-        const int grid = sort ? h->grid_sort : h->grid_move;
-        // a plain FP32 step of a batch without magnetic field launches the mover with the
-        // clock test inline and the one that queues the tests (the draw's code and
-        // registers cost the common path of this variant 6 %; the FP64 form is bound by
-        // its FP64 pipe and the Boris variant holds its registers anyway, so they keep the
-        // test inline).  The step count (and a load since the last step) decides on the
-        // device which of the two runs, so one captured sort cycle serves every cycle.
-        // The partner that returns at once costs about 3 us, more than the 6 % saves
-        // below some 16 M particle slots.  A batch with a subcycled colliding species
-        // (its candidates and tests bunched on its moving steps) keeps the test inline;
-        // subcycled species that never collide, like neutral targets, do not matter.
-        const bool pair = move && !sort && !h->any_mag && h->precision == PIC_FP32 &&
-                          h->total_cap >= h->pair_min && h->pair_ok;
-        a.pair = pair ? 1 : 0;
-        for (int v = 0; v < (pair ? 2 : 1); ++v) {
-            h->kernels += 1;
-            const bool lean = v == 1;
-            // the pair's inline-test partner without subcycling: its own variant and grid
-            const bool gridv = pair && !lean && !h->any_subcycle;
-            const cudaError_t e =
-                h->precision == PIC_FP64
-                    ? launch_move_f64(a, mag, move, h->any_subcycle, h->any_unmag, sort,
-                                      sort ? h->nt_sort : h->nt, grid, h->stream)
-                    : launch_move_f32(a, mag, move, h->any_subcycle, h->any_unmag, sort, lean,
-                                      gridv, sort ? h->nt_sort : h->nt,
-                                      gridv ? h->grid_test : grid, h->stream);
-            CUDA_TRY(h, e);
+        const bool full = move && !sort && full_step(h, h->step_h);
+        const MoveMode mode = full ? MoveMode::kFull : h->mode;
+        const int nt = sort ? h->nt_sort : h->nt;
+        int grid = sort ? h->grid_sort : full ? h->grid_full : h->grid_move;
+        if (!sort) {
+            const int64_t nw = nt / 32;
+            if (h->max_tiles >= h->chunk_rounds * nw * grid && !(mag && h->precision == PIC_FP64))
+                a.chunk = h->precision == PIC_FP64 ? 2 * kMoveChunk : kMoveChunk;
+            const int64_t blocks = (h->max_tiles + nw * a.chunk - 1) / (nw * a.chunk);
+            if (a.chunk > 1 || blocks < grid) grid = (int)std::max<int64_t>(blocks, 1);
         }
+        h->kernels += 1;
+        const cudaError_t e =
+            h->precision == PIC_FP64
+                ? launch_move_f64(a, mag, move, h->any_subcycle, h->any_unmag, sort, mode, nt, grid, h->stream)
+                : launch_move_f32(a, mag, move, h->any_subcycle, h->any_unmag, sort, mode, nt, grid, h->stream);
+        CUDA_TRY(h, e);
+        if (move) h->test_all = false;
     }
     if (sort) {
         Span sp(h, 2);
@@ -739,20 +760,17 @@ int collect_times(pic_handle* h)
 void set_block(pic_handle* h, int nt)
 {
     h->nt = nt;
-    // (FP32: plain steps of a batch with subcycling that the mover pair does not serve run
-    // the variant with subcycling and the inline clock test, built for fewer warps)
-    const bool subtest = h->any_subcycle && !(h->total_cap >= h->pair_min && h->pair_ok);
-    const int bps = h->precision == PIC_FP64 ? move_blocks_per_sm_f64(h->any_mag, false, false, nt)
-                                             : move_blocks_per_sm_f32(h->any_mag, false, false, subtest, false, nt);
-    h->grid_move = h->sms * std::max(bps, 1);
-    const int bts = h->precision == PIC_FP64 ? bps : move_blocks_per_sm_f32(false, false, false, false, true, nt);
-    h->grid_test = h->sms * std::max(bts, 1);
+    const auto per_sm = h->precision == PIC_FP64 ? move_blocks_per_sm_f64 : move_blocks_per_sm_f32;
+    const bool sub = h->any_subcycle;
+    auto grid = [&](MoveMode m) { return h->sms * std::max(per_sm(h->any_mag, sub, false, false, m, nt), 1); };
+    h->grid_full = grid(MoveMode::kFull);
+    // tiles are fetched ahead where a resident warp has several of them
+    h->grid_move = grid(MoveMode::kAhead);
+    h->mode = h->max_tiles >= h->ahead_tiles * h->grid_move * (nt / 32) ? MoveMode::kAhead : MoveMode::kDirect;
+    if (h->mode == MoveMode::kDirect) h->grid_move = grid(MoveMode::kDirect);
     // (the sort step's variant with the y coordinates of 2-D species holds more shared
     // memory a block; its block size is its own)
-    const int bss = h->precision == PIC_FP64
-                        ? move_blocks_per_sm_f64(h->any_mag, true, h->any_sn2d, h->nt_sort)
-                        : move_blocks_per_sm_f32(h->any_mag, true, h->any_sn2d, false, false, h->nt_sort);
-    h->grid_sort = h->sms * std::max(bss, 1);
+    h->grid_sort = h->sms * std::max(per_sm(h->any_mag, sub, true, h->any_sn2d, MoveMode::kDirect, h->nt_sort), 1);
 }
 
 void drop_graphs(pic_handle* h)
@@ -1014,13 +1032,12 @@ int pic_create(const pic_config* cfg, pic_handle** out)
             for (int q = 0; q < P.nproc; ++q)
                 if (P.kind[q] == PIC_PROC_IONIZE) P.product[q] = ip.seg0 + P.product[q];
             slot += P.cap;
+            h->max_tiles += (P.cap + 127) / 128;
             snode += round_up(I.ncells + 1, 4);
             h->max_cap = std::max(h->max_cap, P.cap);
-            // rare-event queue: the collision candidates of a step and the clock tests
-            // that follow them and ionization (about cap x P each; 4x P is reserved),
-            // and the wall hits (a sixteenth of the segment; twice that with a volume
-            // source, whose re-injected particles may have their clock tests queued on
-            // the next step)
+            // rare-event queue: the collision candidates of a step (about cap x P; 4x P is
+            // reserved) and the wall hits (a sixteenth of the segment; twice that with a
+            // volume source)
             {
                 double numax = 0.0;
                 for (int q = 0; q < I.nproc; ++q)
@@ -1060,10 +1077,13 @@ int pic_create(const pic_config* cfg, pic_handle** out)
     }
     h->rare_cap = std::min<int64_t>(h->rare_cap + 65536, std::max<int64_t>(slot, 65536));
     h->total_cap = slot;
-    if (const char* pm = std::getenv("BITPIC_PAIR_MIN_SLOTS")) h->pair_min = std::atoll(pm);
-    for (int i = 0; i < h->ninst; ++i)
-        for (int q = 0; q < h->inst[i].nproc; ++q)
-            if (species_nstep(h->inst[i], h->inst[i].proc[q].species) > 1) h->pair_ok = false;
+    if (const char* v = std::getenv("BITPIC_PAIR_MIN_SLOTS")) h->full_min = std::atoll(v);
+    if (const char* v = std::getenv("BITPIC_AHEAD_TILES")) h->ahead_tiles = std::atoll(v);
+    if (const char* v = std::getenv("BITPIC_CHUNK_ROUNDS")) h->chunk_rounds = std::atoll(v);
+    for (const SegParams& P : h->segh)
+        if (P.collide && std::find(h->collide_nsteps.begin(), h->collide_nsteps.end(), P.nstep) ==
+                             h->collide_nsteps.end())
+            h->collide_nsteps.push_back(P.nstep);
     h->seg_nodes = snode;
     h->inst_nodes = inode;
     h->ev_total = ev;
@@ -1155,7 +1175,6 @@ int pic_create(const pic_config* cfg, pic_handle** out)
     if (rc == PIC_OK) rc = dalloc(h, &h->cell_part, (size_t)h->nseg * h->cell_chunks);
     if (rc == PIC_OK) rc = dalloc(h, &h->err, 1);
     if (rc == PIC_OK) rc = dalloc(h, &h->step_d, 2);
-    if (rc == PIC_OK) rc = dalloc(h, &h->test_all, 1);
     if (rc == PIC_OK) rc = dalloc(h, &h->kin, (size_t)PIC_MAX_SPECIES);
     if (rc) return bail(rc);
 
@@ -1196,7 +1215,6 @@ int pic_create(const pic_config* cfg, pic_handle** out)
     if (e == cudaSuccess) e = z(h->next_id, (size_t)h->ninst * 8);
     if (e == cudaSuccess) e = z(h->err, 4);
     if (e == cudaSuccess) e = z(h->step_d, 16);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->test_all, 1, sizeof(int), s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(h->segd, h->segh.data(), sizeof(SegParams) * h->segh.size(),
                             cudaMemcpyHostToDevice, s);
@@ -1334,8 +1352,6 @@ int load_particles(pic_handle* h, int32_t inst, int32_t species, int64_t n,
     l.precision = h->precision;
     l.next_id = h->next_id + inst;
     CUDA_TRY(h, launch_load(l, s));
-    // a loaded clock may need its test at any step: the next step draws them all inline
-    CUDA_TRY(h, cudaMemsetAsync(h->test_all, 1, sizeof(int), s));
     // the other copy of the segment holds nothing
     CUDA_TRY(h, launch_fill_i32(h->st[1 - h->cur].cell, P.base, P.base + P.cap, -1, s));
     // counts and the next automatic id
@@ -1352,6 +1368,7 @@ int load_particles(pic_handle* h, int32_t inst, int32_t species, int64_t n,
     CUDA_TRY(h, cudaStreamSynchronize(s));
     h->stale = true;
     h->hist_ready = false;
+    h->test_all = true;  // a loaded clock may need its test at any step
     h->fresh_n[si] = n;
     return PIC_OK;
 }
@@ -1447,7 +1464,7 @@ int enqueue_step(pic_handle* h)
 int capture_window(pic_handle* h, int64_t len, pic_handle::Window* w)
 {
     const int c0 = h->cur;
-    const bool hr0 = h->hist_ready;
+    const bool hr0 = h->hist_ready, ta0 = h->test_all;
     const int64_t step0 = h->step_h, k0 = h->kernels;
     CUDA_TRY(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
     int rc = PIC_OK;
@@ -1460,6 +1477,7 @@ int capture_window(pic_handle* h, int64_t len, pic_handle::Window* w)
     h->step_h = step0;
     h->cur = c0;
     h->hist_ready = hr0;
+    h->test_all = ta0;
     h->kernels = k0;
     if (rc != PIC_OK) {
         if (g) cudaGraphDestroy(g);
@@ -1539,9 +1557,24 @@ int pic_step(pic_handle* h, int64_t nsteps)
         const bool graphs = h->graphs && !h->profiling && !h->tune_phase && K > 0 &&
                             h->stream != nullptr;
         if (graphs) {
-            // the steps up to the end of this sort cycle (or of the call) as one graph
+            // a step with the kFull mover falls anywhere in a cycle: it is launched as it is
+            if (full_step(h, h->step_h)) {
+                if ((rc = enqueue_step(h))) return rc;
+                ++n;
+                continue;
+            }
+            // the steps up to the end of this sort cycle (or of the call, or to the next step
+            // with the kFull mover: then not as a graph, which would seldom fit again)
             const int64_t p = h->step_h % K;
-            const int64_t len = std::min<int64_t>(K - p, nsteps - n);
+            int64_t len = std::min<int64_t>(K - p, nsteps - n);
+            int64_t plain = 1;
+            while (plain < len && !full_step(h, h->step_h + plain)) ++plain;
+            if (plain < len) {
+                for (int64_t k = 0; k < plain; ++k)
+                    if ((rc = enqueue_step(h))) return rc;
+                n += plain;
+                continue;
+            }
             const auto key = std::make_tuple(h->cur, p, len, h->hist_ready);
             auto it = h->windows.find(key);
             if (it == h->windows.end()) {
@@ -1554,6 +1587,7 @@ int pic_step(pic_handle* h, int64_t nsteps)
             }
             CUDA_TRY(h, cudaGraphLaunch(it->second.exec, h->stream));
             h->kernels += it->second.kernels;
+            h->test_all = false;
             h->step_h += len;
             h->cur = it->second.end_cur;
             h->hist_ready = it->second.end_hist;
@@ -1845,7 +1879,7 @@ int pic_restore_counters(pic_handle* h, int64_t step, const uint64_t* next_id)
             if (next_id[i] > 0xFFFFFFFFull) return fail(h, PIC_EINVAL, "pic_restore_counters: next_id >= 2^32");
         CUDA_TRY(h, cudaMemcpy(h->next_id, next_id, 8 * (size_t)h->ninst, cudaMemcpyHostToDevice));
     }
-    CUDA_TRY(h, cudaMemset(h->test_all, 1, sizeof(int)));
+    h->test_all = true;
     // which deposits stand depends on the step a subcycled species next moves on
     if (step != h->step_h && h->any_subcycle) h->stale = true;
     h->step_h = step;

@@ -1,9 +1,8 @@
 // events.cuh -- the rare events of a time step, worked through after the mover:
 // null-collision candidates (Section 2: the MCC step of the PIC cycle; elastic,
-// charge-exchange and ionization kinematics), collision-clock tests that the mover
-// variant without the inline test left (a candidate of this same step when the draw
-// says so) and particles that left through an absorbing or source wall (flux and
-// energy counters, re-injection of the volume source).  The mover queues them
+// charge-exchange and ionization kinematics) and particles that left through an
+// absorbing or source wall (flux and energy counters, re-injection of the volume
+// source).  The mover queues them
 // (rare_pack) so that its own loop stays call-free; here one thread takes one queued
 // particle.  Collisions change only velocities, so the mover has already deposited a
 // candidate; a re-injected particle and the children of an ionization are deposited
@@ -18,8 +17,8 @@ namespace bitpic {
 
 // The cell word of a particle in cell j whose next collision event is a clock test on
 // its species' own step m1: the test is drawn here already (word 0 of its counter, the
-// global step of own step m1), so the mover finds the outcome in the clock instead of
-// queueing the test: a candidate g own steps on (g < D), or the next test at the
+// global step of own step m1), so the mover finds the outcome in the clock and its common
+// path holds for the particle: a candidate g own steps on (g < D), or the next test at the
 // species' next multiple of kGapMax (g = D).  Exactly what the test at m1 would set; a
 // species without collisions keeps clock 0.
 __device__ __forceinline__ int test_word(const SegParams& P, uint32_t id, int j, int64_t m1)
@@ -256,9 +255,6 @@ __global__ void __launch_bounds__(128) k_events(const __grid_constant__ MoveArgs
 {
     const unsigned long long n = min(*a.rare_count, (unsigned long long)a.rare_cap);
     const int64_t step = *a.step;
-    // the movers of this step have read it: from the next step on, clocks that need a
-    // test off the common test steps are queued again
-    if (blockIdx.x == 0 && threadIdx.x == 0 && a.test_all) *a.test_all = 0;
     T* const offp = static_cast<T*>(a.off);
     T* const uxp = static_cast<T*>(a.ux);
     T* const uyp = static_cast<T*>(a.uy);
@@ -284,55 +280,22 @@ __global__ void __launch_bounds__(128) k_events(const __grid_constant__ MoveArgs
             const int64_t slot = (int64_t)(e >> 24);
             const SegParams& P = a.seg[s];
             const uint32_t id = a.id[slot];
-            // a clock test needs only the id and the cell word; the state is read when the
-            // particle collides or left through a wall (a candidate and a wall hit need it
-            // in any case: read together with the id, one round trip to memory fewer)
-            T f = T(0), vx = T(0), vy = T(0), vz = T(0);
-            if (kind != kRareTest) {
-                f = offp[slot];
-                vx = uxp[slot];
-                vy = uyp[slot];
-                vz = uzp[slot];
-            }
-            if ((kind == kRareCandidate || kind == kRareTest) &&
-                in_range(a.err, (int)((uint32_t)a.cell[slot] & kCellMask), 0, P.ncells)) {
-                const int j = (int)((uint32_t)a.cell[slot] & kCellMask);
+            // the state is read together with the id: one round trip to memory
+            T f = offp[slot], vx = uxp[slot], vy = uyp[slot], vz = uzp[slot];
+            const int j0 = (int)((uint32_t)a.cell[slot] & kCellMask);
+            if (kind == kRareCandidate && in_range(a.err, j0, 0, P.ncells)) {
                 const uint4 wd = draw(id, step, kRngCollide, P.key0, P.key1);
-                bool now = kind == kRareCandidate;
-                if (!now) {
-                    // the clock test the mover left: word 0 gives the candidate-free run
-                    // from this step, cut at the species' next multiple of kGapMax steps
-                    const int ks = P.nstep;
-                    const int64_t q = ks == 1 ? step + 1 : (step + 1) / ks;
-                    const int dgrid = kGapMax - (int)((q - 1) % kGapMax);
-                    const int g = min(gap_steps(P.gap, P.glog, wd.x), dgrid);
-                    now = g == 0;
-                    // the next event: a test next step after a candidate now, else the
-                    // candidate g steps on, or the test at the grid step
-                    const int64_t mown = q - 1;
-                    a.cell[slot] = (int)((uint32_t)j | clock_bits(g == 0 ? mown + 1 : mown + g,
-                                                                  g > 0 && g < dgrid));
+                const int p = collide<T>(a, P, s, id, step, j0, f, vx, vy, vz, wd.y, wd.z, slot);
+                if (p >= 0) {
+                    uxp[slot] = vx;
+                    uyp[slot] = vy;
+                    uzp[slot] = vz;
+                    ckey = P.inst * kMaxProc + p;
                 }
-                if (now) {
-                    if (kind == kRareTest) {
-                        f = offp[slot];
-                        vx = uxp[slot];
-                        vy = uyp[slot];
-                        vz = uzp[slot];
-                    }
-                    const int p = collide<T>(a, P, s, id, step, j, f, vx, vy, vz, wd.y, wd.z,
-                                             slot);
-                    if (p >= 0) {
-                        uxp[slot] = vx;
-                        uyp[slot] = vy;
-                        uzp[slot] = vz;
-                        ckey = P.inst * kMaxProc + p;
-                    }
-                    // a candidate is followed by a test on the next own step: drawn now
-                    const int ks = P.nstep;
-                    const int64_t q = ks == 1 ? step + 1 : (step + 1) / ks;  // own step q - 1
-                    a.cell[slot] = test_word(P, id, j, q);
-                }
+                // a candidate is followed by a test on the next own step: drawn now
+                const int ks = P.nstep;
+                const int64_t q = ks == 1 ? step + 1 : (step + 1) / ks;  // own step q - 1
+                a.cell[slot] = test_word(P, id, j0, q);
             } else if (kind == kRareWallLow || kind == kRareWallHigh) {
                 int j = kind == kRareWallLow ? -1 : P.ncells;
                 wkey = 2 * s + (kind == kRareWallLow ? 0 : 1);

@@ -8,23 +8,20 @@
 namespace bitpic {
 
 struct MoveArgs;
+enum class MoveMode;
 
 // ---- mover (mover_f32.cu, mover_f64.cu) ---------------------------------------
 // `move` = false deposits the loaded particles without moving them (the density
 // phase of the initial field); `sub`: some species is subcycled; `mixed`: magnetized and
 // unmagnetized instances in one batch; `sort`: the step also sorts the store by cell
-// into the other copy (MoveArgs.cursor, .d*); `lean` (FP32, a plain step of a batch
-// without magnetic field): the variant that queues collision-clock tests for the event
-// kernel instead of drawing them inline; `gridv`: the inline-test partner of the mover
-// pair, which runs only on the steps where every clock tests (without subcycling: the
-// variant that draws a quad's four tests side by side).  Returns the launch error.
+// into the other copy (MoveArgs.cursor, .d*); `mode`: the variant for a time step that does
+// not sort (any gives the same results on any step).  Returns the launch error.
 cudaError_t launch_move_f32(const MoveArgs& a, bool mag, bool move, bool sub, bool mixed,
-                            bool sort, bool lean, bool gridv, int nt, int grid,
-                            cudaStream_t st);
+                            bool sort, MoveMode mode, int nt, int grid, cudaStream_t st);
 cudaError_t launch_move_f64(const MoveArgs& a, bool mag, bool move, bool sub, bool mixed,
-                            bool sort, int nt, int grid, cudaStream_t st);
-// The rare events the mover queued this step (events.cu): collision candidates, clock
-// tests and wall hits, one thread each, `grid` blocks of 128 threads.
+                            bool sort, MoveMode mode, int nt, int grid, cudaStream_t st);
+// The rare events the mover queued this step (events.cu): collision candidates and wall
+// hits, one thread each, `grid` blocks of 128 threads.
 cudaError_t launch_events(const MoveArgs& a, int precision, int grid, cudaStream_t st);
 // Ionizations against neutral particle targets: convert the requested targets into
 // ions (events.cu); one warp per target cell on the step's request list.
@@ -32,11 +29,8 @@ cudaError_t launch_victims(const MoveArgs& a, int precision, int grid, cudaStrea
 // The y drift of 2-D species after the mover (MoveArgs.yp non-null), before the events.
 cudaError_t launch_drift_y(const MoveArgs& a, int precision, int grid, cudaStream_t st);
 // resident blocks per SM of the mover variant (0 on error)
-// subtest: the grid of a batch whose plain steps run the variant with subcycling and the
-// inline clock test (a subcycled colliding species, or a batch below the mover pair's size);
-// gridv: the grid of the pair's inline-test partner without subcycling
-int move_blocks_per_sm_f32(bool mag, bool sort, bool yp, bool subtest, bool gridv, int nt);
-int move_blocks_per_sm_f64(bool mag, bool sort, bool yp, int nt);
+int move_blocks_per_sm_f32(bool mag, bool sub, bool sort, bool yp, MoveMode mode, int nt);
+int move_blocks_per_sm_f64(bool mag, bool sub, bool sort, bool yp, MoveMode mode, int nt);
 
 // ---- field phase and bookkeeping (field.cu) -------------------------------------
 struct FieldArgs {

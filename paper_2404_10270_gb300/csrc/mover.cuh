@@ -35,23 +35,20 @@
 
 namespace bitpic {
 
+// Resident warps per SM the FP32 mover is built for.  With every warp's next tile on its
+// way through shared memory, 32 warps keep HBM busy, and more of them only spread the
+// accesses over more DRAM pages at a time (196.6 M particles: 0.646 ms at 32, 0.651 at 48
+// in 256-thread blocks; 0.69 against 0.76 on a persistent grid).
 #ifndef BITPIC_MOVE_MIN_WARPS
-#define BITPIC_MOVE_MIN_WARPS 48
+#define BITPIC_MOVE_MIN_WARPS 32
 #endif
-constexpr int kMoveMinWarps = BITPIC_MOVE_MIN_WARPS;  // resident warps per SM the mover is built for
-#ifndef BITPIC_MOVE_MIN_WARPS_SUBTEST
-#define BITPIC_MOVE_MIN_WARPS_SUBTEST 40
+constexpr int kMoveMinWarps = BITPIC_MOVE_MIN_WARPS;
+#ifndef BITPIC_MOVE_MIN_WARPS_FULL
+#define BITPIC_MOVE_MIN_WARPS_FULL 32
 #endif
-// the FP32 variant with subcycling and the inline clock test, which runs every step of a
-// batch with a subcycled colliding species: 48 resident warps leave it 40 registers and
-// ~100 B of spills, 40 leave it 48 (measured 2.5 % faster a step on 196.6 M particles)
-constexpr int kMoveMinWarpsSubTest = BITPIC_MOVE_MIN_WARPS_SUBTEST;
-#ifndef BITPIC_MOVE_MIN_WARPS_GRID
-#define BITPIC_MOVE_MIN_WARPS_GRID 32
-#endif
-// the FP32 variant for the steps on which every clock without a candidate tests (GRID):
+// the FP32 variant for the steps on which every clock without a candidate tests (FULL):
 // four draws in flight per lane want registers more than warps
-constexpr int kMoveMinWarpsGrid = BITPIC_MOVE_MIN_WARPS_GRID;
+constexpr int kMoveMinWarpsFull = BITPIC_MOVE_MIN_WARPS_FULL;
 #ifndef BITPIC_MOVE_MIN_WARPS64
 #define BITPIC_MOVE_MIN_WARPS64 32
 #endif
@@ -61,7 +58,7 @@ constexpr int kMoveMinWarps64 = BITPIC_MOVE_MIN_WARPS64;  // the same for the FP
 #endif
 constexpr int kMoveMinWarpsMag = BITPIC_MOVE_MIN_WARPS_MAG;  // the Boris (3V) variant, FP32
 #ifndef BITPIC_MOVE_MIN_WARPS64_MAG
-#define BITPIC_MOVE_MIN_WARPS64_MAG 24
+#define BITPIC_MOVE_MIN_WARPS64_MAG 20
 #endif
 constexpr int kMoveMinWarps64Mag = BITPIC_MOVE_MIN_WARPS64_MAG;  // the Boris variant, FP64
 
@@ -77,6 +74,7 @@ struct MoveArgs {
     int nseg;
     const int64_t* tile_start;          // nseg+1 prefix of tiles
     const int64_t* seg_nmove;           // slots of each segment moved this step
+    int chunk;                          // consecutive tiles a warp of k_move takes at a time
     unsigned long long* seg_n;          // slots in use (appends for created particles)
     unsigned long long* seg_live;       // live particles
     const void* accel;                  // T pairs (A_j, A_{j+1} - A_j), segment node arrays
@@ -106,14 +104,6 @@ struct MoveArgs {
     // scanned counts, by the cell at the start of the step) and writes it there
     unsigned* hist_out;
     unsigned* cursor;
-    // the collision-clock test: on the steps that are multiples of kGapMax every clock
-    // without a candidate tests, and after a load (`test_all` set) any clock may.  With
-    // `pair` set both variants are launched for the step: the one with the test inline
-    // runs on those steps, the one that queues the few other tests for the event kernel
-    // on the rest, and each returns at once on the steps that are not its own (0: the
-    // variant launched runs).
-    int* test_all;
-    int pair;
     int32_t* dcell;
     void* doff;
     void* dux;
@@ -126,6 +116,9 @@ struct MoveArgs {
     void* dyp;
 };
 
+// Variants of the mover for a time step, see k_move.
+enum class MoveMode { kDirect, kAhead, kFull };
+
 template <typename T> struct Prec;
 template <> struct Prec<float> {
     using Q = uint32_t;  // fixed-point charge of one particle (< 2^25)
@@ -134,10 +127,9 @@ template <> struct Prec<float> {
     // Boris vectors t, s of the segment in this precision
     static __device__ __forceinline__ float bt(const SegParams& P, int k) { return P.tf[k]; }
     static __device__ __forceinline__ float bs(const SegParams& P, int k) { return P.sf[k]; }
-    static constexpr int min_warps = kMoveMinWarps;  // memory bound: as many warps as fit
+    static constexpr int min_warps = kMoveMinWarps;
     static constexpr int min_warps_mag = kMoveMinWarpsMag;
-    static constexpr int min_warps_subtest = kMoveMinWarpsSubTest;
-    static constexpr int min_warps_grid = kMoveMinWarpsGrid;
+    static constexpr int min_warps_full = kMoveMinWarpsFull;
     static __device__ __forceinline__ uint64_t qright(float f)
     {
         return (uint64_t)__float2uint_rn(f * 16777216.0f);
@@ -170,6 +162,16 @@ template <> struct Prec<float> {
             j += 1;
         }
     }
+    // The same without the renormalisation: dj cells crossed; true when f' rounded up to
+    // 1 or the velocity is not finite (f' is then a NaN), which move() handles.
+    static __device__ __forceinline__ bool move_fast(float& f, float u, int& dj)
+    {
+        const float xn = f + u;
+        const float fl = floorf(xn);
+        f = xn - fl;
+        dj = (int)fl;
+        return !(f < 1.0f);
+    }
 };
 template <> struct Prec<double> {
     using Q = uint64_t;  // fixed-point charge of one particle (< 2^49)
@@ -179,8 +181,7 @@ template <> struct Prec<double> {
     static __device__ __forceinline__ double bs(const SegParams& P, int k) { return P.s[k]; }
     static constexpr int min_warps = kMoveMinWarps64;  // FP64-pipe bound: registers first
     static constexpr int min_warps_mag = kMoveMinWarps64Mag;
-    static constexpr int min_warps_subtest = kMoveMinWarps64;
-    static constexpr int min_warps_grid = kMoveMinWarps64;
+    static constexpr int min_warps_full = kMoveMinWarps64Mag;
     // rint(f 2^48) for f in [0, 1), ties to even, from the bits: f = m 2^(e-1075), so
     // f 2^48 = m / 2^(1027-e) rounded to nearest even (integer ALU only).
     static __device__ __forceinline__ uint64_t qright(double f)
@@ -249,16 +250,24 @@ template <> struct Prec<double> {
         }
         f = fk;
     }
+    // The common -1 < f' < 2 of the same in two halves.  First f' alone and the cells
+    // crossed, -1, 0 or 1 (true for anything else, which move() handles); then, for the
+    // quad's crossed particles (`cross`, a bit each), the one addition f' - dj.
+    static __device__ __forceinline__ bool move_fast(double& f, double u, int& dj)
+    {
+        f = f + u;
+        const int hi = __double2hiint(f);
+        dj = hi < 0 ? -1 : (hi >= 0x3FF00000 ? 1 : 0);
+        return (hi & 0x7FFFFFFF) >= (hi < 0 ? 0x3FF00000 : 0x40000000);
+    }
 };
 
 // Resident blocks per SM each mover variant is compiled for (its register budget).
-// SUBTEST: the variant with subcycling and the inline clock test; GRID: the variant for
-// the steps on which every clock tests.
-template <typename T, bool MAG, int NT, bool SUBTEST = false, bool GRID = false>
+// FULL: the variant for the steps on which every clock tests.
+template <typename T, bool MAG, int NT, bool FULL = false>
 struct MoveOccupancy {
     static constexpr int warps = MAG ? Prec<T>::min_warps_mag
-                                 : GRID ? Prec<T>::min_warps_grid
-                                 : SUBTEST ? Prec<T>::min_warps_subtest : Prec<T>::min_warps;
+                                 : FULL ? Prec<T>::min_warps_full : Prec<T>::min_warps;
     static constexpr int blocks = warps / (NT / 32) > 0 ? warps / (NT / 32) : 1;
 };
 
@@ -287,28 +296,36 @@ __device__ __forceinline__ void st4(double* p, const double v[4])
     __stcs(reinterpret_cast<double2*>(p) + 1, make_double2(v[2], v[3]));
 }
 
-// Warp-level deposit of four particles per lane.  With Q = rint(f S) the charge of
-// one particle is S - Q on node j and Q on node j+1, so the total on node c is
-//     S n_c - R_c + R_{c-1},   n_c = particles in cell c,  R_c = sum of their Q.
-// The warp forms n_c and R_c for every cell of its range [wmin, wmax]; lane l then
-// owns node wmin + l, takes R_{c-1} from lane l-1 by shuffle, and adds the node total
-// to HBM with one 64-bit reduction (no return value, so nothing waits on it).  A warp
-// whose particles sit in a few cells (the store was sorted recently) forms the sums by
-// register reductions, one round per cell; one whose particles have spread over more
-// cells (late in a sort cycle) adds each lane's runs of equal cells into a window of
-// 32 cells in shared memory (`win`, the warp's own, zero outside this call), which
-// costs the same few instructions whatever the spread; beyond 32 cells every particle
-// goes to HBM on its own.
-// jd = -1 marks an empty slot: as unsigned it is never the minimum of a live cell, as
-// signed never the maximum, and it matches no cell.
+// Warp-level deposit of four particles per lane.  With Q = rint(f S) the charge of one
+// particle is S - Q on node j and Q on node j+1; a tile of 128 particles puts at most
+// 128 S on a node, so a node's sum fits 32 bits (FP64: two halves of 24 bits and up).  The
+// warp forms the sums of the nodes of its range [wmin, wmax + 1]; lane l then owns node
+// wmin + l and adds its sum to HBM with one 64-bit reduction (no return value, so nothing
+// waits on it).  A warp whose particles sit in a few cells (the store was sorted
+// recently) forms them by register reductions, one per node: a lane's shares of node i
+// are S - Q of its particles in cell i and Q of those in cell i-1, which the round before
+// has added up.  One whose particles have spread over more cells (late in a sort cycle)
+// adds each particle's two shares into a window of 32 nodes in shared memory (`win`, the
+// warp's own, zero outside this call; kDepReps copies side by side, a lane's by its
+// number, so that lanes in one cell seldom meet), which costs the same few instructions
+// whatever the spread; beyond 32 nodes every particle goes to HBM on its own.
+// A negative jd marks an empty slot: as unsigned it is never the minimum of a live cell,
+// as signed never the maximum, and it matches no cell.
 // gdep null (OPT variants): only the counts, for a species whose deposit stands.
-constexpr int kDepLoopCells = 6;  // register reductions up to this many cells
+// Register reductions up to this many cells (FP64: one more, its window costs four shared
+// atomics a particle).  196.6 M particles, FP32, 256-thread blocks: 0.644 ms at 2, 0.655 at
+// 3, 0.662 at 5; FP64, 512-thread blocks: 1.475 at 2, 1.435 at 3, 1.444 at 5.
+template <typename Q>
+struct DepLoop {
+    static constexpr int cells = sizeof(Q) == 4 ? 2 : 3;
+};
+constexpr int kDepReps = 4;
 
-// Words of a warp's deposit window: 32 counts and 32 charge sums (FP64: the 48-bit
-// charges as two 24-bit halves; a half summed over a tile of 128 stays below 2^31).
+// Words of a warp's deposit window: 32 nodes of kDepReps copies (FP64: low halves, then
+// high halves; a half summed over a tile of 128 stays below 2^32).
 template <typename Q>
 struct DepWin {
-    static constexpr int words = sizeof(Q) == 4 ? 64 : 96;
+    static constexpr int words = 32 * kDepReps * (sizeof(Q) / 4);
 };
 
 // Clear the warp's window (once, before its first deposit).
@@ -321,6 +338,15 @@ __device__ __forceinline__ void dep_win_clear(uint32_t* win)
     __syncwarp();
 }
 
+// Sum of a lane's node copies in the window, which are cleared.
+__device__ __forceinline__ uint32_t dep_win_take(uint32_t* win)
+{
+    uint4* const p = reinterpret_cast<uint4*>(win) + (threadIdx.x & 31);
+    const uint4 v = *p;
+    *p = make_uint4(0u, 0u, 0u, 0u);
+    return (v.x + v.y) + (v.z + v.w);
+}
+
 template <typename Q, bool OPT = false>
 __device__ __forceinline__ void warp_deposit(const int jd[4], const Q qr[4],
                                              unsigned long long S,
@@ -328,117 +354,85 @@ __device__ __forceinline__ void warp_deposit(const int jd[4], const Q qr[4],
                                              unsigned* __restrict__ ghist,
                                              uint32_t* __restrict__ win)
 {
+    static_assert(kDepReps == 4, "dep_win_take reads a node's copies as one uint4");
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    unsigned lmin = 0xFFFFFFFFu;
-    int lmax = -1;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        lmin = min(lmin, (unsigned)jd[k]);
-        lmax = max(lmax, jd[k]);
-    }
-    const unsigned wminu = __reduce_min_sync(FULL, lmin);
-    if (wminu == 0xFFFFFFFFu) return;  // no live particle in the tile
-    const int wmin = (int)wminu;
+    const unsigned lmin = min(min((unsigned)jd[0], (unsigned)jd[1]), min((unsigned)jd[2], (unsigned)jd[3]));
+    const int lmax = max(max(jd[0], jd[1]), max(jd[2], jd[3]));
+    const int wmin = (int)__reduce_min_sync(FULL, lmin);
+    if (wmin < 0) return;  // no live particle in the tile
     const int wmax = __reduce_max_sync(FULL, lmax);
     const int ncell = wmax - wmin + 1;
     if (ncell < 32) {
-        unsigned long long myR = 0;  // R_c of cell wmin + lane
-        uint32_t myn = 0;            // n_c of cell wmin + lane
-        if (ncell <= kDepLoopCells) {
-            for (int i = 0; i < ncell; ++i) {
-                const int cidx = wmin + i;
-                uint32_t n = 0;
-                if (sizeof(Q) == 4) {
-                    uint32_t r = 0;  // at most 128 x 2^24 < 2^32
+        if (!OPT || gdep) {
+            unsigned long long tot = 0;  // the sum of node wmin + lane
+            if (ncell <= DepLoop<Q>::cells) {
+                Q left[4], carry = 0;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const bool in = jd[k] == cidx;
-                        r += in ? (uint32_t)qr[k] : 0u;
-                        n += in ? 1u : 0u;
-                    }
-                    const uint32_t tr = __reduce_add_sync(FULL, r);
-                    const uint32_t tn = __reduce_add_sync(FULL, n);
-                    if (lane == i) {
-                        myR = tr;
-                        myn = tn;
-                    }
-                } else {
-                    // 48-bit charges: reduce the high and low 24-bit halves separately
-                    uint32_t lo = 0, hi = 0;
+                for (int k = 0; k < 4; ++k) left[k] = (Q)S - qr[k];
+#pragma unroll 1
+                for (int i = 0; i <= ncell; ++i) {
+                    Q l = carry, rr = 0;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const bool in = jd[k] == cidx;
-                        const uint64_t q = in ? (uint64_t)qr[k] : 0ull;
-                        lo += (uint32_t)(q & 0xFFFFFFu);
-                        hi += (uint32_t)(q >> 24);
-                        n += in ? 1u : 0u;
-                    }
-                    const uint32_t tl = __reduce_add_sync(FULL, lo);
-                    const uint32_t th = __reduce_add_sync(FULL, hi);
-                    const uint32_t tn = __reduce_add_sync(FULL, n);
-                    if (lane == i) {
-                        myR = ((unsigned long long)th << 24) + tl;
-                        myn = tn;
-                    }
-                }
-            }
-        } else {
-            // each run of equal cells among the lane's four (consecutive) particles is
-            // added to the window once
-            uint32_t n = 0, lo = 0, hi = 0;
-            int cur = -1;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (jd[k] != cur) {
-                    if (cur >= 0) {
-                        atomicAdd(win + (cur - wmin), n);
-                        atomicAdd(win + 32 + (cur - wmin), lo);
-                        if (sizeof(Q) == 8) atomicAdd(win + 64 + (cur - wmin), hi);
-                    }
-                    cur = jd[k];
-                    n = lo = hi = 0u;
-                }
-                if (jd[k] >= 0) {
-                    n += 1u;
+                    for (int k = 0; k < 4; ++k)
+                        if (jd[k] == wmin + i) {
+                            l += left[k];
+                            rr += qr[k];
+                        }
+                    carry = rr;
                     if (sizeof(Q) == 4) {
-                        lo += (uint32_t)qr[k];
+                        const uint32_t t = __reduce_add_sync(FULL, (uint32_t)l);
+                        if (lane == i) tot = t;
                     } else {
-                        lo += (uint32_t)((uint64_t)qr[k] & 0xFFFFFFu);
-                        hi += (uint32_t)((uint64_t)qr[k] >> 24);
+                        const uint32_t lo = __reduce_add_sync(FULL, (uint32_t)((uint64_t)l & 0xFFFFFFu));
+                        const uint32_t hi = __reduce_add_sync(FULL, (uint32_t)((uint64_t)l >> 24));
+                        if (lane == i) tot = ((unsigned long long)hi << 24) + lo;
                     }
                 }
+            } else {
+                uint32_t* const w = win + (lane & (kDepReps - 1));
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (jd[k] < 0) continue;
+                    uint32_t* const p = w + kDepReps * (jd[k] - wmin);
+                    const Q l = (Q)S - qr[k];
+                    if (sizeof(Q) == 4) {
+                        atomicAdd(p, (uint32_t)l);
+                        atomicAdd(p + kDepReps, (uint32_t)qr[k]);
+                    } else {
+                        atomicAdd(p, (uint32_t)((uint64_t)l & 0xFFFFFFu));
+                        atomicAdd(p + kDepReps, (uint32_t)((uint64_t)qr[k] & 0xFFFFFFu));
+                        atomicAdd(p + 32 * kDepReps, (uint32_t)((uint64_t)l >> 24));
+                        atomicAdd(p + 33 * kDepReps, (uint32_t)((uint64_t)qr[k] >> 24));
+                    }
+                }
+                __syncwarp();
+                tot = dep_win_take(win);
+                if (sizeof(Q) == 8) tot += (unsigned long long)dep_win_take(win + 32 * kDepReps) << 24;
+                __syncwarp();
             }
-            if (cur >= 0) {
-                atomicAdd(win + (cur - wmin), n);
-                atomicAdd(win + 32 + (cur - wmin), lo);
-                if (sizeof(Q) == 8) atomicAdd(win + 64 + (cur - wmin), hi);
-            }
-            __syncwarp();
-            myn = win[lane];
-            myR = win[32 + lane];
-            if (sizeof(Q) == 8) myR += (unsigned long long)win[64 + lane] << 24;
-            win[lane] = 0u;  // (lanes past the range read and write zeros)
-            win[32 + lane] = 0u;
-            if (sizeof(Q) == 8) win[64 + lane] = 0u;
-            __syncwarp();
-        }
-        const unsigned long long prevR = __shfl_up_sync(FULL, myR, 1);
-        if (lane <= ncell && (!OPT || gdep)) {
-            const unsigned long long tot =
-                S * (unsigned long long)myn - myR + (lane > 0 ? prevR : 0ull);
+            // (lanes past the range hold zeros)
             if (tot != 0) atomicAdd(gdep + wmin + lane, tot);
         }
-        // the particles per cell, for a sort in the next step
-        if (ghist && lane < ncell && myn != 0u) atomicAdd(ghist + wmin + lane, myn);
+        if (ghist) {  // the particles per cell, for a sort in the next step
+            uint32_t n = 0;
+#pragma unroll 1
+            for (int i = 0; i < ncell; ++i) {
+                uint32_t t = 0;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) t += __popc(__ballot_sync(FULL, jd[k] == wmin + i));
+                if (lane == i) n = t;
+            }
+            if (n != 0u) atomicAdd(ghist + wmin + lane, n);
+        }
     } else {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             if (jd[k] >= 0) {
-                const unsigned long long l = S - (unsigned long long)qr[k], r = qr[k];
+                const unsigned long long l = S - (unsigned long long)qr[k], rr = qr[k];
                 if (!OPT || gdep) {
                     atomicAdd(gdep + jd[k], l);
-                    atomicAdd(gdep + jd[k] + 1, r);
+                    atomicAdd(gdep + jd[k] + 1, rr);
                 }
                 if (ghist) atomicAdd(ghist + jd[k], 1u);
             }
@@ -493,145 +487,356 @@ __device__ __forceinline__ void sort_write(const MoveArgs& a, const int64_t to[4
     }
 }
 
-// Steps 1-5 of the time step for the four particles of one quad (a lane's share of
-// a tile): gather, push, move, walls, collision clock.  c, f, u* hold the quad's
-// state on entry and its new state on exit (cell word -1: left through a wall).  The
-// masks get one bit per quad position: collision candidate (cand), absorbed at the
-// low or high wall (wlo, whi), clock test left to the event kernel (tst), cell word
-// changed (chg).  mown is the species' own index of this step (its clock's time),
-// dgrid the own steps to its next multiple of kGapMax.  The id of a test draw comes
-// from idq (SORT: already loaded) or from the store at `slot`; PRE: the test's
-// candidate-free run (before the cut at dgrid) is already in gq.
-template <typename T, bool MAG, bool SORT, bool TEST, bool PRE = false>
-__device__ __forceinline__ void quad_physics(const MoveArgs& a, const SegParams& P, bool smag,
-                                             int64_t step, int64_t mown, int dgrid, int64_t slot,
-                                             const uint32_t idq[4], int c[4], T f[4], T ux[4],
-                                             T uy[4], T uz[4], unsigned& cand, unsigned& wlo,
-                                             unsigned& whi, unsigned& tst, unsigned& chg,
-                                             const int* gq = nullptr)
+// The push of one particle (step 2) in cells per own step, acc the acceleration at its
+// position: u += acc, or the Boris rotation.
+template <typename T, bool MAG>
+__device__ __forceinline__ void push(const SegParams& P, bool smag, T acc, T& ux, T& uy, T& uz)
+{
+    if (!MAG || !smag) {
+        ux = ux + acc;
+        return;
+    }
+    const T half = T(0.5) * acc;
+    const T t0 = Prec<T>::bt(P, 0), t1 = Prec<T>::bt(P, 1), t2 = Prec<T>::bt(P, 2);
+    const T s0 = Prec<T>::bs(P, 0), s1 = Prec<T>::bs(P, 1), s2 = Prec<T>::bs(P, 2);
+    const T mx = ux + half, my = uy, mz = uz;
+    // v' = v + v x t, v+ = v + v' x s, each component as two fused
+    // multiply-adds (m_x + m_y t_z - m_z t_y = fma(m_y, t_z, fma(-m_z, t_y, m_x)))
+    const T px = Prec<T>::fma_(my, t2, Prec<T>::fma_(-mz, t1, mx));
+    const T py = Prec<T>::fma_(mz, t0, Prec<T>::fma_(-mx, t2, my));
+    const T pz = Prec<T>::fma_(mx, t1, Prec<T>::fma_(-my, t0, mz));
+    const T qx = Prec<T>::fma_(py, s2, Prec<T>::fma_(-pz, s1, mx));
+    const T qy = Prec<T>::fma_(pz, s0, Prec<T>::fma_(-px, s2, my));
+    const T qz = Prec<T>::fma_(px, s1, Prec<T>::fma_(-py, s0, mz));
+    ux = qx + half;
+    uy = qy;
+    uz = qz;
+}
+
+// A tile's state on its way through shared memory: each lane copies its own quad (16
+// bytes an access) with cp.async one tile ahead and reads it back itself, so a warp keeps
+// a whole tile's loads in flight while it works on the tile before, without registers
+// for them.  Once its instructions had gone from 448 to 289 a tile the FP32 mover waited
+// for HBM with 46 warps' loads in flight (0.730 ms for 196.6 M particles); with the ring
+// and kMoveChunk (engine.cu) it takes 0.64-0.65 ms, 6.1 TB/s of the 20 B a particle it
+// moves in fact.  One stage: the cell words, off, ux (and uy, uz) of a warp's tile.
+template <typename T, bool MAG>
+struct TileRing {
+    static constexpr int words = 128 + (MAG ? 4 : 2) * 128 * (int)(sizeof(T) / 4);  // one stage
+    static constexpr size_t bytes(int nt) { return (size_t)(nt / 32) * 2 * words * 4; }
+};
+// Dynamic shared memory of a block of the mover: the rings of the variants that fetch ahead.
+template <typename T, bool MAG, MoveMode MODE>
+constexpr size_t ring_bytes(int nt)
+{
+    return MODE == MoveMode::kAhead ? TileRing<T, MAG>::bytes(nt) : 0;
+}
+// L2 policy of streamed reads: evict first (as the 128-bit loads' hint).
+__device__ __forceinline__ uint64_t stream_policy()
+{
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ void copy16(uint32_t dst, const void* src, uint64_t policy)
+{
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
+                 "l"(policy)
+                 : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void copy_wait_1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
+// The lane's share of one array of a tile: four values of type V.
+template <typename V>
+__device__ __forceinline__ void copy_quad(uint32_t dst, const V* src, uint64_t policy)
+{
+    const uint32_t d = dst + (threadIdx.x & 31) * 4 * sizeof(V);
+    copy16(d, src, policy);
+    if (sizeof(V) == 8) copy16(d + 16, src + 2, policy);
+}
+__device__ __forceinline__ void take_quad(const uint32_t* p, float v[4])
+{
+    const float4 t = reinterpret_cast<const float4*>(p)[threadIdx.x & 31];
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+__device__ __forceinline__ void take_quad(const uint32_t* p, double v[4])
+{
+    const double2* q = reinterpret_cast<const double2*>(p) + 2 * (threadIdx.x & 31);
+    const double2 a = q[0], b = q[1];
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
+
+// Put a particle on the step's list for the event kernel.
+__device__ __forceinline__ void queue_rare(const MoveArgs& a, int s, int64_t slot, uint32_t kind)
+{
+    const unsigned long long e = atomicAdd(a.rare_count, 1ull);
+    if (e < (unsigned long long)a.rare_cap) a.rare[e] = rare_pack(slot, s, kind);
+    else set_error(a.err, kErrEvents);
+}
+
+// Steps 1-5 of the time step for one live particle: gather, push, move, walls,
+// collision clock.  c, f, u* hold its state on entry and its new state on exit (cell
+// word -1: left through a wall).  mown is the species' own index of this step (its
+// clock's time), dgrid the own steps to its next multiple of kGapMax; run() gives the
+// candidate-free run of this step's test draw.  Returns what the event kernel has to do
+// with the particle (kRareCandidate, kRareWallLow, kRareWallHigh) or -1.
+template <typename T, bool MAG, typename Run>
+__device__ __forceinline__ int particle_step(const MoveArgs& a, const SegParams& P, bool smag,
+                                             int64_t mown, int dgrid, Run run, int& c, T& f, T& ux,
+                                             T& uy, T& uz)
 {
     using T2 = typename Prec<T>::T2;
-    const T2* const accp = static_cast<const T2*>(a.accel);
     const int N = P.ncells;
-    const int bc = P.bc;
-    const int collides = P.collide;
-    const uint32_t key0 = P.key0, key1 = P.key1;
-    const int64_t node0 = P.node;
+    int j = (int)((uint32_t)c & kCellMask);
+    uint32_t clk = (uint32_t)c >> kClockShift;
+    if (!in_range(a.err, j, 0, N)) {  // (bounds-checked build only)
+        c = -1;
+        return -1;
+    }
+    // 1. gather (Listing 7) from the node pair (A_j, A_{j+1} - A_j)
+    const T2 pr = __ldg(static_cast<const T2*>(a.accel) + P.node + j);
+    T fk = f;
+    // 2. push
+    push<T, MAG>(P, smag, Prec<T>::fma_(fk, pr.y, pr.x), ux, uy, uz);
+    if (!Prec<T>::finite(ux)) set_error(a.err, kErrNonFinite);
+    // 3. move (Listing 7: x += nstep*vx, x the in-cell offset)
+    Prec<T>::move(fk, ux, j);
+    f = fk;
+    // 4. walls: periodic wrap here; an absorbed or re-injected particle
+    // leaves the store and the event kernel takes over
+    if (j < 0 || j >= N) {
+        if (P.bc != PIC_BC_PERIODIC) {
+            c = -1;
+            return j < 0 ? (int)kRareWallLow : (int)kRareWallHigh;
+        }
+        j %= N;
+        if (j < 0) j += N;
+    }
+    // 5. null collision.  The candidate steps of a particle form a
+    // Bernoulli(P) sequence; its clock names the own step of its next event
+    // step.  At an event step without a pending candidate (a test), Philox word
+    // 0 gives the candidate-free run g from this step, cut at the next multiple
+    // of 127 (D steps away): g = 0 candidate now, g < D a candidate g steps
+    // later, g = D none before then.  The cut puts the tests of all particles on
+    // the same steps.  Candidates go to the event kernel.  Between events the
+    // clock, and so the word, does not change.
+    int ev = -1;
+    if (P.collide && (clk & kClockDue) == (uint32_t)(mown & (int64_t)kClockDue)) {
+        if (clk & kClockPending) {
+            ev = (int)kRareCandidate;
+            // a test next step (the event kernel draws it when it takes the
+            // candidate and puts its outcome in the clock)
+            clk = (uint32_t)((mown + 1) & (int64_t)kClockDue);
+        } else {
+            const int g = min(run(), dgrid);
+            if (g == 0) ev = (int)kRareCandidate;
+            const int64_t due = g == 0 ? mown + 1 : mown + g;
+            clk = (uint32_t)(due & (int64_t)kClockDue) | (g > 0 && g < dgrid ? kClockPending : 0u);
+        }
+    }
+    c = (int)((uint32_t)j | (clk << kClockShift));
+    return ev;
+}
+
+// The FP64 additions of a tile's crossed particles (move_fast), `cross` a bit per quad
+// position.  A tenth of the electrons cross a cell edge in a step, so with an addition
+// per quad position nearly every warp would issue all four for a few lanes each; the FP64
+// pipe, which takes a warp's addition at the same price however few its lanes, is this
+// form's limit.  The crossed values are brought together in `scr` (32 doubles of the
+// warp) and added 32 at a time: one addition a tile.  True when a sum rounded up to 1.
+__device__ __forceinline__ bool add_crossed(double f[4], unsigned cross, double* scr)
+{
+    const unsigned FULL = 0xffffffffu;
+    if (!__any_sync(FULL, cross != 0u)) return false;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    int at[4], n = 0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        if (c[k] < 0) continue;
-        const int cw = c[k];
-        int j = (int)((uint32_t)c[k] & kCellMask);
-        uint32_t clk = (uint32_t)c[k] >> kClockShift;
-        if (!in_range(a.err, j, 0, N)) {  // (bounds-checked build only)
-            c[k] = -1;
-            chg |= 1u << k;
-            continue;
+        const unsigned b = __ballot_sync(FULL, cross >> k & 1u);
+        at[k] = (cross >> k & 1u) ? n + __popc(b & lt) : -1;
+        n += __popc(b);
+    }
+    bool odd = false;
+#pragma unroll 1
+    for (int r0 = 0; r0 < n; r0 += 32) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if ((unsigned)(at[k] - r0) < 32u && at[k] >= 0) scr[at[k] - r0] = f[k];
+        __syncwarp();
+        if (r0 + lane < n) {
+            const double x = scr[lane];
+            scr[lane] = x + __hiloint2double(__double2hiint(x) < 0 ? 0x3FF00000 : (int)0xBFF00000u, 0);
         }
-        // 1. gather (Listing 7) from the node pair (A_j, A_{j+1} - A_j)
-        const T2 pr = __ldg(accp + node0 + j);
-        T fk = f[k];
-        const T acc = Prec<T>::fma_(fk, pr.y, pr.x);
-        // 2. push
-        if (!MAG || !smag) {
-            ux[k] = ux[k] + acc;
-        } else {
-            const T half = T(0.5) * acc;
-            const T t0 = Prec<T>::bt(P, 0), t1 = Prec<T>::bt(P, 1), t2 = Prec<T>::bt(P, 2);
-            const T s0 = Prec<T>::bs(P, 0), s1 = Prec<T>::bs(P, 1), s2 = Prec<T>::bs(P, 2);
-            const T mx = ux[k] + half, my = uy[k], mz = uz[k];
-            // v' = v + v x t, v+ = v + v' x s, each component as two fused
-            // multiply-adds (m_x + m_y t_z - m_z t_y = fma(m_y, t_z, fma(-m_z, t_y, m_x)))
-            const T px = Prec<T>::fma_(my, t2, Prec<T>::fma_(-mz, t1, mx));
-            const T py = Prec<T>::fma_(mz, t0, Prec<T>::fma_(-mx, t2, my));
-            const T pz = Prec<T>::fma_(mx, t1, Prec<T>::fma_(-my, t0, mz));
-            const T qx = Prec<T>::fma_(py, s2, Prec<T>::fma_(-pz, s1, mx));
-            const T qy = Prec<T>::fma_(pz, s0, Prec<T>::fma_(-px, s2, my));
-            const T qz = Prec<T>::fma_(px, s1, Prec<T>::fma_(-py, s0, mz));
-            ux[k] = qx + half;
-            uy[k] = qy;
-            uz[k] = qz;
-        }
-        if (!Prec<T>::finite(ux[k])) set_error(a.err, kErrNonFinite);
-        // 3. move (Listing 7: x += nstep*vx, x the in-cell offset)
-        Prec<T>::move(fk, ux[k], j);
-        f[k] = fk;
-        // 4. walls: periodic wrap here; an absorbed or re-injected particle
-        // leaves the store and the event kernel takes over
-        if (j < 0 || j >= N) {
-            if (bc == PIC_BC_PERIODIC) {
-                j %= N;
-                if (j < 0) j += N;
-            } else {
-                if (j < 0) wlo |= 1u << k; else whi |= 1u << k;
-                c[k] = -1;
-                chg |= 1u << k;
-                continue;
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if ((unsigned)(at[k] - r0) < 32u && at[k] >= 0) {
+                f[k] = scr[at[k] - r0];
+                odd |= __double2hiint(f[k]) == 0x3FF00000;
             }
-        }
-        // 5. null collision.  The candidate steps of a particle form a
-        // Bernoulli(P) sequence; its clock names the own step of its next event
-        // step.  At an event step without a pending candidate (a test), Philox word
-        // 0 gives the candidate-free run g from this step, cut at the next multiple
-        // of 127 (D steps away): g = 0 candidate now, g < D a candidate g steps
-        // later, g = D none before then.  The cut puts the tests of all particles on
-        // the same steps, so a warp runs them together.  Candidates go to the event
-        // kernel.  Between events the clock, and so the word, does not change.
-        if (collides && (clk & kClockDue) == (uint32_t)(mown & (int64_t)kClockDue)) {
-            if (clk & kClockPending) {
-                cand |= 1u << k;
-                // a test next step (the event kernel draws it when it takes the
-                // candidate and puts its outcome in the clock)
-                clk = (uint32_t)((mown + 1) & (int64_t)kClockDue);
-            } else if (!TEST) {
-                // a test off the common test steps (the first clock of an ionization
-                // product, whose id the event kernel did not know yet, or of a loaded
-                // particle): the event kernel draws it, with this step's counter, and
-                // sets the clock
-                tst |= 1u << k;
-            } else {
-                // a test step: the id is read only here
-                int g;
-                if (PRE) {
-                    g = min(gq[k], dgrid);
-                } else {
-                    const uint32_t idk = SORT ? idq[k] : __ldg(a.id + slot + k);
-                    const uint4 w = draw(idk, step, kRngCollide, key0, key1);
-                    g = min(gap_steps(P.gap, P.glog, w.x), dgrid);
-                }
-                if (g == 0) cand |= 1u << k;
-                const int64_t due = g == 0 ? mown + 1 : mown + g;
-                clk = (uint32_t)(due & (int64_t)kClockDue) | (g > 0 && g < dgrid ? kClockPending : 0u);
+        __syncwarp();
+    }
+    return odd;
+}
+__device__ __forceinline__ bool add_crossed(float*, unsigned, double*) { return false; }
+// Words of that scratch.
+template <typename T>
+struct CrossScratch {
+    static constexpr int words = sizeof(T) == 8 ? 64 : 0;
+};
+
+// The segment constants of the common path, held in registers across the tiles of a
+// segment.  A particle's clock is due when (c ^ due) & clkmask == 0; a species without
+// collisions gets a pattern that only an empty slot (bit 31) matches.
+struct SegFast {
+    int N;
+    uint32_t clkmask, due;
+    __device__ __forceinline__ void set(const SegParams& P, int64_t mown)
+    {
+        N = P.ncells;
+        clkmask = P.collide ? kClockDue << kClockShift : 0x80000000u;
+        due = P.collide ? ((uint32_t)mown & kClockDue) << kClockShift : 0x80000000u;
+    }
+};
+
+// Steps 1-5 for the four particles of one quad (a lane's share of a tile), the common
+// case: live particles that stay inside the walls.  The mover is bound by its
+// instructions as much as by HBM, so this runs without branches: the cell is the word's
+// low bits, so the new word is the old one plus the cells crossed.  due: a clock of the
+// quad is due (quad_due).  Returns true when a particle of the quad is not of that kind
+// (a wall, an offset that rounded up to 1, a velocity that is not finite): the whole quad is then done over by rare_quad from the state in memory, which must not
+// have been written before.
+template <typename T, bool MAG>
+__device__ __forceinline__ bool quad_fast(const SegParams& P, const SegFast& F, bool smag,
+                                          const typename Prec<T>::T2* __restrict__ accn, int c[4],
+                                          T f[4], T ux[4], T uy[4], T uz[4], bool& moved, bool& due,
+                                          double* scr)
+{
+    using T2 = typename Prec<T>::T2;
+    // an empty slot is given a particle at rest in the first cell, its clock not due, and
+    // emptied again below
+    unsigned empty = 0;
+    if ((c[0] | c[1] | c[2] | c[3]) < 0) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (c[k] < 0) {
+                empty |= 1u << k;
+                c[k] = (int)((F.due ^ (1u << kClockShift)) & (kClockDue << kClockShift));
+                f[k] = T(0.5);
+                ux[k] = T(0);
+                if (MAG) uy[k] = uz[k] = T(0);
             }
+    }
+    T2 pr[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)  // (the clamp only bounds a corrupted word)
+        pr[k] = __ldg(accn + min((uint32_t)c[k] & kCellMask, (uint32_t)F.N));
+    bool rare = false;
+    int crossed = 0;
+    unsigned cross = 0;
+    due = false;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        push<T, MAG>(P, smag, Prec<T>::fma_(f[k], pr[k].y, pr[k].x), ux[k], uy[k], uz[k]);
+        int dj;
+        rare |= Prec<T>::move_fast(f[k], ux[k], dj);
+        rare |= (uint32_t)((int)((uint32_t)c[k] & kCellMask) + dj) >= (uint32_t)F.N;
+        due |= (((uint32_t)c[k] ^ F.due) & F.clkmask) == 0u;
+        c[k] += dj;
+        crossed |= dj;
+        if (sizeof(T) == 8 && dj != 0) cross |= 1u << k;
+    }
+    rare |= add_crossed(f, cross, scr);
+    if (empty) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (empty >> k & 1) c[k] = -1;
+    }
+    moved = crossed != 0;
+    return rare;
+}
+
+// A quad of the common path with a due clock: one bit per pending collision candidate,
+// whose clocks are set to the test that follows (the event kernel draws it when it takes
+// the candidate); -1 when a clock tests, which is left to rare_quad.
+__device__ __forceinline__ int quad_due(const SegFast& F, int c[4])
+{
+    constexpr uint32_t pend = kClockPending << kClockShift;
+    const uint32_t mask = F.clkmask | pend, next = (F.due + (1u << kClockShift)) & F.clkmask;
+    bool test = false;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) test |= c[k] >= 0 && (((uint32_t)c[k] ^ F.due) & mask) == 0u;
+    if (test) return -1;
+    int cand = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (c[k] >= 0 && (((uint32_t)c[k] ^ F.due) & mask) == pend) {
+            cand |= 1 << k;
+            c[k] = (int)(((uint32_t)c[k] & kCellMask) | next);
         }
-        c[k] = (int)((uint32_t)j | (clk << kClockShift));
-        if (c[k] != cw) chg |= 1u << k;
+    return cand;
+}
+
+// The species' own index of step `step` (its clock's time) and the own steps to its next
+// multiple of kGapMax.
+__device__ __forceinline__ void own_time(const SegParams& P, int64_t step, int64_t& mown, int& dgrid)
+{
+    mown = P.nstep == 1 ? step : (step + 1) / P.nstep - 1;
+    dgrid = kGapMax - (int)(mown % kGapMax);
+}
+
+// One particle of a quad the common path left, from the state in memory at slot g:
+// steps 1-5, its deposit (and count) straight to HBM, its event queued at slot `to` (where
+// it lies after the step; -1: none, nothing is queued).  The caller writes the state.
+template <typename T, bool MAG>
+__device__ __forceinline__ void rare_particle(const MoveArgs& a, const SegParams& P, int s,
+                                              bool smag, int64_t step, int64_t mown, int dgrid,
+                                              int64_t g, int64_t to, int& c, T& f, T& ux, T& uy,
+                                              T& uz)
+{
+    f = static_cast<const T*>(a.off)[g];
+    ux = static_cast<const T*>(a.ux)[g];
+    if (MAG && smag) {
+        uy = static_cast<const T*>(a.uy)[g];
+        uz = static_cast<const T*>(a.uz)[g];
+    }
+    const int ev = particle_step<T, MAG>(
+        a, P, smag, mown, dgrid,
+        [&] { return gap_steps(P.gap, P.glog, draw(__ldg(a.id + g), step, kRngCollide, P.key0, P.key1).x); },
+        c, f, ux, uy, uz);
+    if (ev >= 0 && to >= 0) queue_rare(a, s, to, (uint32_t)ev);
+    const int j = (int)((uint32_t)c & kCellMask);
+    if (c >= 0 && in_range(a.err, j, 0, P.ncells)) {
+        const unsigned long long qr = Prec<T>::qright(f);
+        atomicAdd(a.dep + P.node + j, Prec<T>::S - qr);
+        atomicAdd(a.dep + P.node + j + 1, qr);
+        if (a.hist_out) atomicAdd(a.hist_out + P.node + j, 1u);
     }
 }
 
-// Queue the quad's rare events for the event kernel (a few lanes of a few tiles per
-// step).  at[k]: the slot the particle occupies after this step (-1: none, nothing is
-// queued for it).
-__device__ __forceinline__ void queue_rare(const MoveArgs& a, int s, unsigned cand, unsigned wlo,
-                                           unsigned whi, unsigned tst, const int64_t at[4])
+// A quad the common path left (plain step): its particles one by one, in place.
+template <typename T, bool MAG>
+__device__ __forceinline__ void rare_quad(const MoveArgs& a, int s, bool smag, int64_t step,
+                                          int64_t slot)
 {
-    const unsigned ev = cand | wlo | whi | tst;
-    if (!ev) return;
-    unsigned long long e = atomicAdd(a.rare_count, (unsigned long long)__popc(ev));
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const unsigned bit = 1u << k;
-        if (!(ev & bit)) continue;
-        const uint32_t kind = (cand & bit) ? kRareCandidate
-                              : (tst & bit) ? kRareTest
-                              : (wlo & bit) ? kRareWallLow : kRareWallHigh;
-        if (at[k] < 0) {
-            // refused destination (capacity error latched): nothing to queue
-        } else if (e < (unsigned long long)a.rare_cap)
-            a.rare[e] = rare_pack(at[k], s, kind);
-        else
-            set_error(a.err, kErrEvents);
-        ++e;
+    const SegParams& P = a.seg[s];
+    int64_t mown;
+    int dgrid;
+    own_time(P, step, mown, dgrid);
+#pragma unroll 1
+    for (int64_t g = slot; g < slot + 4; ++g) {
+        int c = a.cell[g];
+        if (c < 0) continue;
+        T f, ux, uy = T(0), uz = T(0);
+        rare_particle<T, MAG>(a, P, s, smag, step, mown, dgrid, g, g, c, f, ux, uy, uz);
+        a.cell[g] = c;
+        static_cast<T*>(a.off)[g] = f;
+        static_cast<T*>(a.ux)[g] = ux;
+        if (MAG && smag) {
+            static_cast<T*>(a.uy)[g] = uy;
+            static_cast<T*>(a.uz)[g] = uz;
+        }
     }
 }
 
@@ -641,85 +846,124 @@ __device__ __forceinline__ void queue_rare(const MoveArgs& a, int s, unsigned ca
 // keeps many tiles' loads in flight.  The gather reads each particle's node pair with
 // one vector load (the node arrays are small and stay in L1/L2).  The loop is free of
 // calls; walls and collision candidates are queued for the event kernel.
-// SUB: some species of the batch is subcycled (else every segment moves every step and
-// the clock grid is the global one, computed once).  MIXED (with MAG): the batch mixes
-// magnetized and unmagnetized instances, so the push is chosen per segment.
-// TEST: the collision-clock test (a Philox draw and a table search) runs inline;
-// without it a particle whose clock needs a test is queued for the event kernel, which
-// keeps the common path free of the draw's code and registers.  A segment that rests on
-// this step (subcycling, a neutral particle target) keeps its deposit, so its tiles are
-// skipped, or only counted per cell on the step before a sort: the 30,011-cell plasma
-// with ions moved every fourth step (42 M particles, FP32) went from 212 to 183 us a step.  (The step that
-// ends a sort cycle runs k_move_sort below instead.)
-template <typename T, int NT, bool MAG, bool MOVE, bool SUB, bool MIXED, bool TEST,
-          bool GRID = false>
-__global__ void __launch_bounds__(NT, MoveOccupancy<T, MAG, NT, MOVE && SUB && TEST, GRID>::blocks)
+// SUB: some species of the batch is subcycled (else every segment moves every step).
+// MIXED (with MAG): the batch mixes magnetized and unmagnetized instances, so the push is
+// chosen per segment.  MODE: kDirect loads a tile when its turn comes, for batches whose
+// warps have a tile or two (a ring of two 16 KB stages a block buys nothing there and its
+// set-up costs 1.5 us a step) and for the FP64 Boris form (4.6 KB a tile, bound by the FP64
+// pipe); kAhead fetches one tile ahead (TileRing); kFull is the variant of large batches
+// for the steps on which the clocks of a whole species test (the multiples of kGapMax, the
+// first step after a load):
+// the quad's ids are read with its state and its four draws and table lookups go side by
+// side before the physics; the other steps' variant leaves such quads, one particle at a
+// time, to rare_quad, which gives the same results.  A segment that rests on this step
+// (subcycling, a neutral particle target) keeps its deposit, so its tiles are skipped, or
+// only counted per cell on the step before a sort: the 30,011-cell plasma with ions moved
+// every fourth step (42 M particles, FP32) went from 212 to 183 us a step.  (The step
+// that ends a sort cycle runs k_move_sort below instead.)
+template <typename T, int NT, bool MAG, bool MOVE, bool SUB, bool MIXED, MoveMode MODE>
+__global__ void __launch_bounds__(NT, MoveOccupancy<T, MAG, NT, MODE == MoveMode::kFull>::blocks)
 k_move(const __grid_constant__ MoveArgs a)
 {
     using Q = typename Prec<T>::Q;
+    using T2 = typename Prec<T>::T2;
+    constexpr bool PF = MODE == MoveMode::kAhead, FULL = MODE == MoveMode::kFull;
     const int lane = threadIdx.x & 31;
     T* const offp = static_cast<T*>(a.off);
     T* const uxp = static_cast<T*>(a.ux);
     T* const uyp = static_cast<T*>(a.uy);
     T* const uzp = static_cast<T*>(a.uz);
     const int64_t step = MOVE ? *a.step : 0;
-    if (MOVE && a.pair) {
-        // every clock without a candidate tests on the multiples of kGapMax (a pair is
-        // launched only when every colliding species moves on every step)
-        const bool tstep = step % kGapMax == 0 || *a.test_all != 0;
-        if (tstep != TEST) return;
-    }
-    __shared__ uint32_t s_dwin[NT / 32][DepWin<Q>::words];  // the warps' deposit windows
+    // the warps' deposit windows and (FP64) scratch of add_crossed
+    __shared__ __align__(16) uint32_t s_dwin[NT / 32][DepWin<Q>::words + CrossScratch<T>::words];
     uint32_t* const dwin = s_dwin[threadIdx.x >> 5];
+    double* const scr = reinterpret_cast<double*>(dwin + DepWin<Q>::words);
     dep_win_clear<Q>(dwin);
-    const int64_t total = a.tile_start[a.nseg];
-    const int64_t wstride = (int64_t)gridDim.x * (NT / 32);
-    int s = 0;                         // segment of the previous tile (tiles only increase)
-    int64_t s_begin = 0, s_end = -1;   // its tiles
-    bool moves = MOVE;                 // the segment moves this step (subcycling)
-    bool smag = MAG;                   // the segment's instance is magnetized
-    // steps (of the segment's species) to the next multiple of kGapMax
-    int dgrid = kGapMax - (int)(step % kGapMax);
-    int64_t mown = step;  // the segment's own index of this step (its clock's time)
-    for (int64_t tile = (int64_t)blockIdx.x * (NT / 32) + (threadIdx.x >> 5); tile < total;
-         tile += wstride) {
-        if (tile >= s_end) {
-            s = advance_segment(a.tile_start, a.nseg, s, tile);
-            s_begin = __ldg(a.tile_start + s);
-            s_end = __ldg(a.tile_start + s + 1);
-            // in a batch that mixes magnetized and unmagnetized instances, the latter
-            // keep the plain push (and never touch uy, uz), as they would alone
-            if (MAG && MIXED) smag = a.seg[s].mag != 0;
-            if (MOVE && SUB) {
-                // a species with subcycling factor K moves on the steps n with
-                // (n+1) mod K = 0 (all species meet at the multiples of K dt); its
-                // collision clock counts its own steps, (n+1)/K - 1, and at the multiples
-                // of kGapMax of those every clock without a candidate tests
-                const int ks = a.seg[s].nstep;
-                const int64_t q = ks == 1 ? step + 1 : (step + 1) / ks;
-                moves = ks == 1 || q * ks == step + 1;
-                dgrid = kGapMax - (int)((q - 1) % kGapMax);
-                mown = q - 1;
-                // a species that rests keeps its deposit: the warp goes on with its first
-                // tile past the segment
-                if (!moves && !a.hist_out) {
-                    tile += ((s_end - 1 - tile) / wstride) * wstride;
-                    continue;
-                }
+    // (fewer than 2^31 tiles: 2^38 particles would not fit)
+    const int total = (int)a.tile_start[a.nseg];
+    // the tile ahead: its segment (tiles only increase) with that segment's last tile + 1 and
+    // slots (ahead0: as if tile 0 were its), and the slot of the lane's quad
+    int tile = (blockIdx.x * (NT / 32) + (threadIdx.x >> 5)) * a.chunk, left = a.chunk - 1;
+    int sa = 0, sa_end = -1;
+    int64_t ahead0 = 0, ahead_end = 0, ahead = 0;
+    const auto next = [&]() {
+        ++tile;
+        if (--left < 0) {  // on to the warp's next chunk
+            left = a.chunk - 1;
+            tile += (int)(gridDim.x * (NT / 32) - 1) * a.chunk;
+        }
+    };
+    const auto look = [&]() {
+        while (tile < total && tile >= sa_end) {
+            sa = advance_segment(a.tile_start, a.nseg, sa, tile);
+            sa_end = (int)__ldg(a.tile_start + sa + 1);
+            const SegParams& P = a.seg[sa];
+            ahead0 = P.base - 128 * __ldg(a.tile_start + sa) + 4 * lane;
+            ahead_end = P.base + a.seg_nmove[sa];
+            // a species that rests keeps its deposit: the warp goes on with its first tile
+            // past the segment
+            if (MOVE && SUB && !a.hist_out && !moves_on(P, step))
+                while (tile < sa_end) next();
+        }
+        ahead = ahead0 + (int64_t)tile * 128;
+    };
+    extern __shared__ __align__(16) uint32_t s_ring[];
+    constexpr int SW = TileRing<T, MAG>::words;
+    uint32_t* const ring = s_ring + (threadIdx.x >> 5) * 2 * SW;
+    const uint32_t ring_at = PF ? (uint32_t)__cvta_generic_to_shared(ring) : 0u;
+    const uint64_t policy = PF ? stream_policy() : 0ull;
+    const auto fetch = [&](int stage) {
+        if (tile < total && ahead < ahead_end) {
+            const uint32_t d = ring_at + stage * SW * 4;
+            copy_quad(d, a.cell + ahead, policy);
+            copy_quad(d + 512, offp + ahead, policy);
+            copy_quad(d + 512 + 128 * sizeof(T), uxp + ahead, policy);
+            if (MAG) {
+                copy_quad(d + 512 + 256 * sizeof(T), uyp + ahead, policy);
+                copy_quad(d + 512 + 384 * sizeof(T), uzp + ahead, policy);
             }
         }
-        const SegParams& P = a.seg[s];
-        const int64_t node0 = P.node;
-        const int64_t quad = (tile - s_begin) * 32 + lane;
-        const int64_t nq = a.seg_nmove[s] >> 2;
-        const int64_t slot = P.base + 4 * quad;
-        const bool act = quad < nq && in_range(a.err, slot + 3, P.base, P.base + P.cap);
-
+        copy_commit();
+    };
+    int s = -1;             // segment of the current tile
+    int64_t node0 = 0;      // its nodes
+    bool moves = MOVE;      // it moves this step (subcycling)
+    bool smag = MAG;        // its instance is magnetized
+    SegFast F = {0, 0u, 0u};
+    look();
+    if (PF) fetch(0);
+    for (int stage = 0; tile < total; stage ^= 1) {
+        const int64_t slot = ahead;
+        const bool act = slot < ahead_end && in_range(a.err, slot + 3, a.seg[sa].base, a.seg[sa].base + a.seg[sa].cap);
+        const bool fresh = s != sa;  // the segment's first tile here
+        s = sa;
+        if (fresh && MAG && MIXED) {
+            // in a batch that mixes magnetized and unmagnetized instances, the latter
+            // keep the plain push (and never touch uy, uz), as they would alone
+            smag = a.seg[s].mag != 0;
+        }
+        if (fresh && MOVE && SUB) moves = moves_on(a.seg[s], step);
         int c[4] = {-1, -1, -1, -1};
         T f[4] = {T(0), T(0), T(0), T(0)}, ux[4] = {T(0), T(0), T(0), T(0)};
         T uy[4] = {T(0), T(0), T(0), T(0)}, uz[4] = {T(0), T(0), T(0), T(0)};
         uint32_t idq[4] = {0u, 0u, 0u, 0u};
-        if (act) {
+        if (PF) {
+            next();
+            look();
+            fetch(stage ^ 1);
+            copy_wait_1();
+            if (act) {
+                const uint32_t* const w = ring + stage * SW;
+                const int4 cc = reinterpret_cast<const int4*>(w)[lane];
+                c[0] = cc.x; c[1] = cc.y; c[2] = cc.z; c[3] = cc.w;
+                take_quad(w + 128, f);
+                take_quad(w + 128 + 32 * sizeof(T), ux);
+                if (MAG) {
+                    take_quad(w + 128 + 64 * sizeof(T), uy);
+                    take_quad(w + 128 + 96 * sizeof(T), uz);
+                }
+            }
+        } else if (act) {
             const int4 cc = __ldcs(reinterpret_cast<const int4*>(a.cell + slot));
             c[0] = cc.x; c[1] = cc.y; c[2] = cc.z; c[3] = cc.w;
             ld4(offp + slot, f);
@@ -728,31 +972,70 @@ k_move(const __grid_constant__ MoveArgs a)
                 ld4(uyp + slot, uy);
                 ld4(uzp + slot, uz);
             }
-            if (GRID) {
+            if (FULL) {
                 const uint4 ii = __ldcs(reinterpret_cast<const uint4*>(a.id + slot));
                 idq[0] = ii.x; idq[1] = ii.y; idq[2] = ii.z; idq[3] = ii.w;
             }
         }
-        // GRID: every clock without a candidate tests on this step, so the quad's four
-        // draws (and their table lookups) go first, side by side, while the state loads
-        // are in flight; a clock that does not test ignores its result
-        int gq[4] = {0, 0, 0, 0};
-        if (GRID && P.collide) {
-            uint32_t w[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) w[k] = draw(idq[k], step, kRngCollide, P.key0, P.key1).x;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) gq[k] = gap_steps(P.gap, P.glog, w[k]);
+        if (!PF) {
+            next();
+            look();
         }
+        if (fresh) {
+            const SegParams& P = a.seg[s];
+            node0 = P.node;
+            int64_t mown;
+            int dgrid;
+            own_time(P, step, mown, dgrid);
+            F.set(P, mown);
+        }
+        bool rare = false;
         if (MOVE && (!SUB || moves)) {
-            unsigned cand = 0, wlo = 0, whi = 0, tst = 0, chg = 0;
-            quad_physics<T, MAG, false, TEST, GRID>(a, P, smag, step, mown, dgrid, slot, idq, c, f,
-                                                    ux, uy, uz, cand, wlo, whi, tst, chg, gq);
+            const SegParams& P = a.seg[s];
+            bool moved = false;
+            if (FULL) {
+                // a clock that does not test ignores its draw
+                int gq[4] = {0, 0, 0, 0};
+                if (P.collide) {
+                    uint32_t w[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        w[k] = draw(idq[k], step, kRngCollide, P.key0, P.key1).x;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) gq[k] = gap_steps(P.gap, P.glog, w[k]);
+                }
+                int64_t mown;
+                int dgrid;
+                own_time(P, step, mown, dgrid);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (c[k] < 0) continue;
+                    const int cw = c[k];
+                    const int ev = particle_step<T, MAG>(a, P, smag, mown, dgrid,
+                                                         [&] { return gq[k]; }, c[k], f[k], ux[k],
+                                                         uy[k], uz[k]);
+                    if (ev >= 0) queue_rare(a, s, slot + k, (uint32_t)ev);
+                    moved |= c[k] != cw;
+                }
+            } else {
+                bool due;
+                rare = quad_fast<T, MAG>(P, F, smag, static_cast<const T2*>(a.accel) + node0, c, f,
+                                         ux, uy, uz, moved, due, scr) && act;
+                if (due && act && !rare) {
+                    const int cand = quad_due(F, c);
+                    rare = cand < 0;
+                    moved = true;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (!rare && (cand >> k & 1)) queue_rare(a, s, slot + k, kRareCandidate);
+                }
+            }
             // the cell words go back only where one of them changed (a cell crossing, a
             // wall, a collision event: a few per cent of the particles a step), decided
             // per 32-byte sector (two lanes) so that memory sees whole sectors
-            const bool wcell = (chg | __shfl_xor_sync(0xffffffffu, chg, 1)) != 0u;
-            if (act) {
+            const int chg = moved ? 1 : 0;
+            const bool wcell = (chg | __shfl_xor_sync(0xffffffffu, chg, 1)) != 0;
+            if (act && !rare) {
                 if (wcell)
                     __stcs(reinterpret_cast<int4*>(a.cell + slot), make_int4(c[0], c[1], c[2], c[3]));
                 st4(offp + slot, f);
@@ -762,21 +1045,21 @@ k_move(const __grid_constant__ MoveArgs a)
                     st4(uzp + slot, uz);
                 }
             }
-            const int64_t at[4] = {slot, slot + 1, slot + 2, slot + 3};
-            queue_rare(a, s, cand, wlo, whi, tst, at);
         }
-        // 6. deposit of the (new) positions; an empty slot (cell word < 0) gets jd = -1
+        // 6. deposit of the (new) positions; an empty slot has jd < 0 (bit 31 of its word), and
+        // so have the quads left to rare_quad
         int jd[4];
         Q qr[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            jd[k] = (c[k] >> 31) | (int)((uint32_t)c[k] & kCellMask);
-            if (jd[k] >= 0 && !in_range(a.err, jd[k], 0, P.ncells)) jd[k] = -1;
-            qr[k] = c[k] >= 0 ? (Q)Prec<T>::qright(f[k]) : (Q)0;
+            jd[k] = rare ? -1 : (int)((uint32_t)c[k] & (kCellMask | 0x80000000u));
+            if (kChecked && jd[k] >= 0 && !in_range(a.err, jd[k], 0, a.seg[s].ncells)) jd[k] = -1;
+            qr[k] = (Q)Prec<T>::qright(f[k]);
         }
         warp_deposit<Q, MOVE && SUB>(jd, qr, Prec<T>::S,
                                      MOVE && SUB && !moves ? nullptr : a.dep + node0,
                                      a.hist_out ? a.hist_out + node0 : nullptr, dwin);
+        if (!FULL && rare) rare_quad<T, MAG>(a, s, smag, step, slot);
     }
 }
 
@@ -814,6 +1097,7 @@ __global__ void __launch_bounds__(NT, MoveOccupancy<T, true, NT>::blocks)
 k_move_sort(const __grid_constant__ MoveArgs a)
 {
     using Q = typename Prec<T>::Q;
+    using T2 = typename Prec<T>::T2;
     constexpr int NW = NT / 32, C = NW * 128;
     const unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -835,8 +1119,10 @@ k_move_sort(const __grid_constant__ MoveArgs a)
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    __shared__ uint32_t s_dwin[NW][DepWin<Q>::words];  // the warps' deposit windows
+    // the warps' deposit windows and (FP64) scratch of add_crossed
+    __shared__ __align__(16) uint32_t s_dwin[NW][DepWin<Q>::words + CrossScratch<T>::words];
     uint32_t* const dwin = s_dwin[warp];
+    double* const scr = reinterpret_cast<double*>(dwin + DepWin<Q>::words);
     dep_win_clear<Q>(dwin);
     T* const offp = static_cast<T*>(a.off);
     T* const uxp = static_cast<T*>(a.ux);
@@ -847,8 +1133,7 @@ k_move_sort(const __grid_constant__ MoveArgs a)
     int s = 0;
     int64_t s_begin = 0, s_end = -1;
     bool moves = true, smag = MAG;
-    int dgrid = kGapMax - (int)(step % kGapMax);
-    int64_t mown = step;  // the segment's own index of this step (its clock's time)
+    SegFast F = {0, 0u, 0u};
     // every warp of the block walks the same chunks, so the barriers below match
     int parity = 0;
     for (int64_t chunk = blockIdx.x; chunk * NW < total; chunk += gridDim.x, parity ^= 1) {
@@ -862,13 +1147,11 @@ k_move_sort(const __grid_constant__ MoveArgs a)
             s_begin = __ldg(a.tile_start + s);
             s_end = __ldg(a.tile_start + s + 1);
             if (MAG && MIXED) smag = a.seg[s].mag != 0;
-            if (SUB) {
-                const int ks = a.seg[s].nstep;
-                const int64_t q = ks == 1 ? step + 1 : (step + 1) / ks;
-                moves = ks == 1 || q * ks == step + 1;
-                dgrid = kGapMax - (int)((q - 1) % kGapMax);
-                mown = q - 1;
-            }
+            if (SUB) moves = moves_on(a.seg[s], step);
+            int64_t mown;
+            int dgrid;
+            own_time(a.seg[s], step, mown, dgrid);
+            F.set(a.seg[s], mown);
         }
         const SegParams& P = a.seg[s];
         const int64_t quad = (tile - s_begin) * 32 + lane;
@@ -931,8 +1214,9 @@ k_move_sort(const __grid_constant__ MoveArgs a)
             bmax = __reduce_max_sync(FULL, mx);
         }
         const bool staged = one && bseg >= 0 && bmax - bmin < kSortSpan;
-        unsigned cand = 0, wlo = 0, whi = 0, tst = 0, chg = 0;  // (the sort writes every word)
-        int64_t to[4] = {-1, -1, -1, -1};
+        bool rare = false, moved = false;
+        int cand = 0;  // collision candidates of a quad that is not rare
+        const T2* const accn = static_cast<const T2*>(a.accel) + P.node;
         if (staged) {
             const SegParams& B = a.seg[bseg];
             // rank of each particle among the chunk's particles of its start cell: equal
@@ -976,17 +1260,26 @@ k_move_sort(const __grid_constant__ MoveArgs a)
                     run += v[i];
                 }
             }
-            if (!SUB || moves)
-                quad_physics<T, MAG, true, true>(a, P, smag, step, mown, dgrid, slot, idq, c, f,
-                                                 ux, uy, uz, cand, wlo, whi, tst, chg);
+            if (!SUB || moves) {
+                bool due;
+                rare = quad_fast<T, MAG>(P, F, smag, accn, c, f, ux, uy, uz, moved, due, scr) && act;
+                if (due && act && !rare) {
+                    cand = quad_due(F, c);
+                    rare = cand < 0;
+                }
+            }
             if (threadIdx.x < kSortSpan) gb[threadIdx.x] = gres;
             __syncthreads();
-            // stage every particle at its place in the chunk's cell order
+            // stage every particle at its place in the chunk's cell order; a quad the
+            // common path left is staged where it lay and put right below
+            int pk[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
+                pk[k] = -1;
                 if (key[k] < 0) continue;
                 const int p = pre[key[k]] + rank[k];
                 if (!in_range(a.err, p, 0, C)) continue;  // (bounds-checked build only)
+                pk[k] = p;
                 s_off[p] = f[k];
                 s_ux[p] = ux[k];
                 s_uy[p] = uy[k];
@@ -995,10 +1288,33 @@ k_move_sort(const __grid_constant__ MoveArgs a)
                 s_id[p] = idq[k];
                 if (YP) s_yp[p] = static_cast<const T*>(a.yp)[slot + k];
                 const int64_t r = (int64_t)gb[key[k]] + rank[k];
-                to[k] = r < B.cap ? B.base + r : -1;
                 s_dst[p] = r < B.cap ? (uint32_t)r : 0xFFFFFFFFu;
+                if (!rare && (cand >> k & 1) && r < B.cap)
+                    queue_rare(a, bseg, B.base + r, kRareCandidate);
             }
-            queue_rare(a, bseg, cand, wlo, whi, tst, to);
+            if (rare) {
+                int64_t mown;
+                int dgrid;
+                own_time(B, step, mown, dgrid);
+#pragma unroll 1
+                for (int k = 0; k < 4; ++k) {
+                    const int p = k == 0 ? pk[0] : k == 1 ? pk[1] : k == 2 ? pk[2] : pk[3];
+                    if (p < 0) continue;
+                    int ck = a.cell[slot + k];
+                    T fk, xk, yk = s_uy[p], zk = s_uz[p];
+                    const uint32_t d = s_dst[p];
+                    rare_particle<T, MAG>(a, B, bseg, smag, step, mown, dgrid, slot + k,
+                                          d == 0xFFFFFFFFu ? (int64_t)-1 : B.base + (int64_t)d, ck,
+                                          fk, xk, yk, zk);
+                    s_cell[p] = ck;
+                    s_off[p] = fk;
+                    s_ux[p] = xk;
+                    if (MAG && smag) {
+                        s_uy[p] = yk;
+                        s_uz[p] = zk;
+                    }
+                }
+            }
             // (read before the barrier: the next chunk clears the counts after it)
             const int ntot = pre[kSortSpan - 1] + cnt[kSortSpan - 1];
             __syncthreads();
@@ -1035,9 +1351,15 @@ k_move_sort(const __grid_constant__ MoveArgs a)
                 if (j0[k] >= 0 && lane == __ffs(grp[k]) - 1)
                     rbase[k] = atomicAdd(a.cursor + P.node + kk, (unsigned)__popc(grp[k]));
             }
-            if (!SUB || moves)
-                quad_physics<T, MAG, true, true>(a, P, smag, step, mown, dgrid, slot, idq, c, f,
-                                                 ux, uy, uz, cand, wlo, whi, tst, chg);
+            if (!SUB || moves) {
+                bool due;
+                rare = quad_fast<T, MAG>(P, F, smag, accn, c, f, ux, uy, uz, moved, due, scr) && act;
+                if (due && act && !rare) {
+                    cand = quad_due(F, c);
+                    rare = cand < 0;
+                }
+            }
+            int64_t to[4];
             sort_destinations(a, P, grp, rbase, had, to);
             sort_write<T>(a, to, c, f, ux, uy, uz, idq);
             if (YP) {  // the y coordinates go along
@@ -1046,7 +1368,34 @@ k_move_sort(const __grid_constant__ MoveArgs a)
                     if (to[k] >= 0)
                         static_cast<T*>(a.dyp)[to[k]] = static_cast<const T*>(a.yp)[slot + k];
             }
-            queue_rare(a, s, cand, wlo, whi, tst, to);
+            if (!rare && cand != 0) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if ((cand >> k & 1) && to[k] >= 0) queue_rare(a, s, to[k], kRareCandidate);
+            }
+            if (rare) {
+                // put right what the common path left, in the slots just written
+                int64_t mown;
+                int dgrid;
+                own_time(P, step, mown, dgrid);
+#pragma unroll 1
+                for (int k = 0; k < 4; ++k) {
+                    const int64_t g = k == 0 ? to[0] : k == 1 ? to[1] : k == 2 ? to[2] : to[3];
+                    int ck = a.cell[slot + k];
+                    if (ck < 0) continue;
+                    T fk, xk, yk = T(0), zk = T(0);
+                    rare_particle<T, MAG>(a, P, s, smag, step, mown, dgrid, slot + k, g, ck, fk, xk,
+                                          yk, zk);
+                    if (g < 0) continue;
+                    a.dcell[g] = ck;
+                    static_cast<T*>(a.doff)[g] = fk;
+                    static_cast<T*>(a.dux)[g] = xk;
+                    if (MAG && smag) {
+                        static_cast<T*>(a.duy)[g] = yk;
+                        static_cast<T*>(a.duz)[g] = zk;
+                    }
+                }
+            }
         }
         // 6. deposit of the new positions (that of a segment that rests stands)
         if (SUB && !moves) continue;
@@ -1054,9 +1403,9 @@ k_move_sort(const __grid_constant__ MoveArgs a)
         Q qr[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            jd[k] = (c[k] >> 31) | (int)((uint32_t)c[k] & kCellMask);
-            if (jd[k] >= 0 && !in_range(a.err, jd[k], 0, P.ncells)) jd[k] = -1;
-            qr[k] = c[k] >= 0 ? (Q)Prec<T>::qright(f[k]) : (Q)0;
+            jd[k] = rare ? -1 : (int)((uint32_t)c[k] & (kCellMask | 0x80000000u));
+            if (kChecked && jd[k] >= 0 && !in_range(a.err, jd[k], 0, P.ncells)) jd[k] = -1;
+            qr[k] = (Q)Prec<T>::qright(f[k]);
         }
         warp_deposit<Q>(jd, qr, Prec<T>::S, a.dep + P.node, nullptr, dwin);
     }

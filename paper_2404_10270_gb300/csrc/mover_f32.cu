@@ -5,73 +5,93 @@
 namespace bitpic {
 
 namespace {
-template <int NT, bool SUB, bool TEST>
+// One launch of a variant with the shared memory of its ring.
+template <int NT, bool MAG, bool MOVE, bool SUB, bool MIXED, MoveMode MODE>
+cudaError_t launch(const MoveArgs& a, int grid, cudaStream_t st)
+{
+    k_move<float, NT, MAG, MOVE, SUB, MIXED, MODE><<<grid, NT, ring_bytes<float, MAG, MODE>(NT), st>>>(a);
+    return cudaGetLastError();
+}
+
+template <int NT, bool SUB, MoveMode MODE>
 cudaError_t go_sub(const MoveArgs& a, bool mag, bool mixed, int grid, cudaStream_t st)
 {
-    if (!mag)
-        k_move<float, NT, false, true, SUB, false, TEST><<<grid, NT, 0, st>>>(a);
-    else if (mixed)
-        k_move<float, NT, true, true, SUB, true, TEST><<<grid, NT, 0, st>>>(a);
-    else
-        k_move<float, NT, true, true, SUB, false, TEST><<<grid, NT, 0, st>>>(a);
-    return cudaGetLastError();
+    if (!mag) return launch<NT, false, true, SUB, false, MODE>(a, grid, st);
+    constexpr MoveMode M = MODE;
+    return mixed ? launch<NT, true, true, SUB, true, M>(a, grid, st)
+                 : launch<NT, true, true, SUB, false, M>(a, grid, st);
+}
+
+template <int NT, bool SUB>
+cudaError_t go_mode(const MoveArgs& a, bool mag, bool mixed, MoveMode mode, int grid, cudaStream_t st)
+{
+    if (mode == MoveMode::kFull) return go_sub<NT, SUB, MoveMode::kFull>(a, mag, mixed, grid, st);
+    if (mode == MoveMode::kAhead) return go_sub<NT, SUB, MoveMode::kAhead>(a, mag, mixed, grid, st);
+    return go_sub<NT, SUB, MoveMode::kDirect>(a, mag, mixed, grid, st);
 }
 
 template <int NT>
 cudaError_t go(const MoveArgs& a, bool mag, bool move, bool sub, bool mixed, bool sort,
-               bool lean, bool gridv, int grid, cudaStream_t st)
+               MoveMode mode, int grid, cudaStream_t st)
 {
-    if (!move) {
-        k_move<float, NT, false, false, false, false, true><<<grid, NT, 0, st>>>(a);
-        return cudaGetLastError();
-    }
+    if (!move) return launch<NT, false, false, false, false, MoveMode::kDirect>(a, grid, st);
     if (sort) return launch_sort_step<float, NT>(a, mag, sub, mixed, grid, st);
-    if (gridv && !lean && !mag && !sub) {
-        k_move<float, NT, false, true, false, false, true, true><<<grid, NT, 0, st>>>(a);
-        return cudaGetLastError();
-    }
-    if (lean && !mag) {
-        if (sub)
-            k_move<float, NT, false, true, true, false, false><<<grid, NT, 0, st>>>(a);
-        else
-            k_move<float, NT, false, true, false, false, false><<<grid, NT, 0, st>>>(a);
-        return cudaGetLastError();
-    }
-    if (sub) return go_sub<NT, true, true>(a, mag, mixed, grid, st);
-    return go_sub<NT, false, true>(a, mag, mixed, grid, st);
+    return sub ? go_mode<NT, true>(a, mag, mixed, mode, grid, st)
+               : go_mode<NT, false>(a, mag, mixed, mode, grid, st);
+}
+
+// Resident blocks per SM; also raises the variant's shared-memory limit (a block's rings
+// pass 48 KB), outside any stream capture.
+template <int NT, bool MAG, bool SUB, bool MIXED, MoveMode MODE>
+int resident_one()
+{
+    const auto k = k_move<float, NT, MAG, true, SUB, MIXED, MODE>;
+    const int sm = (int)ring_bytes<float, MAG, MODE>(NT);
+    int n = 0;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, NT, sm);
+    return e == cudaSuccess ? n : 0;
+}
+template <int NT, bool SUB, MoveMode MODE>
+int resident(bool mag)
+{
+    if (!mag) return resident_one<NT, false, SUB, false, MODE>();
+    constexpr MoveMode M = MODE;
+    if (resident_one<NT, true, SUB, true, M>() == 0) return 0;
+    return resident_one<NT, true, SUB, false, M>();
+}
+template <int NT, bool SUB>
+int resident_mode(bool mag, MoveMode mode)
+{
+    if (mode == MoveMode::kFull) return resident<NT, SUB, MoveMode::kFull>(mag);
+    if (mode == MoveMode::kAhead) return resident<NT, SUB, MoveMode::kAhead>(mag);
+    return resident<NT, SUB, MoveMode::kDirect>(mag);
 }
 
 template <int NT>
-int occupancy(bool mag, bool sort, bool yp, bool subtest, bool gridv)
+int occupancy(bool mag, bool sub, bool sort, bool yp, MoveMode mode)
 {
     if (sort) return sort_step_blocks_per_sm<float, NT>(mag, yp);
-    int n = 0;
-    const cudaError_t e =
-        gridv ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_move<float, NT, false, true, false, false, true, true>, NT, 0)
-        : mag ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_move<float, NT, true, true, false, false, true>, NT, 0)
-        : subtest ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_move<float, NT, false, true, true, false, true>, NT, 0)
-                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_move<float, NT, false, true, false, false, true>, NT, 0);
-    return e == cudaSuccess ? n : 0;
+    return sub ? resident_mode<NT, true>(mag, mode) : resident_mode<NT, false>(mag, mode);
 }
 }  // namespace
 
 cudaError_t launch_move_f32(const MoveArgs& a, bool mag, bool move, bool sub, bool mixed,
-                            bool sort, bool lean, bool gridv, int nt, int grid,
-                            cudaStream_t st)
+                            bool sort, MoveMode mode, int nt, int grid, cudaStream_t st)
 {
     switch (nt) {
-        case 128: return go<128>(a, mag, move, sub, mixed, sort, lean, gridv, grid, st);
-        case 512: return go<512>(a, mag, move, sub, mixed, sort, lean, gridv, grid, st);
-        default: return go<256>(a, mag, move, sub, mixed, sort, lean, gridv, grid, st);
+        case 128: return go<128>(a, mag, move, sub, mixed, sort, mode, grid, st);
+        case 512: return go<512>(a, mag, move, sub, mixed, sort, mode, grid, st);
+        default: return go<256>(a, mag, move, sub, mixed, sort, mode, grid, st);
     }
 }
 
-int move_blocks_per_sm_f32(bool mag, bool sort, bool yp, bool subtest, bool gridv, int nt)
+int move_blocks_per_sm_f32(bool mag, bool sub, bool sort, bool yp, MoveMode mode, int nt)
 {
     switch (nt) {
-        case 128: return occupancy<128>(mag, sort, yp, subtest, gridv);
-        case 512: return occupancy<512>(mag, sort, yp, subtest, gridv);
-        default: return occupancy<256>(mag, sort, yp, subtest, gridv);
+        case 128: return occupancy<128>(mag, sub, sort, yp, mode);
+        case 512: return occupancy<512>(mag, sub, sort, yp, mode);
+        default: return occupancy<256>(mag, sub, sort, yp, mode);
     }
 }
 
