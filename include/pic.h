@@ -314,8 +314,8 @@ PIC_API int pic_bounds_probe(void* stream);
  *   z       host array of nspecies integers: species charge q_s w_s = z_s * delta;
  *   eps0    vacuum permittivity;  E  device array of ncells+1 doubles (output);
  *   stream  borrowed cudaStream_t (NULL = default stream); the call only enqueues.
- * Allocates nothing: its scratch (one 128-bit sum per node) is a static device array
- * of the library, 1 MB on every GPU that loads it, held until the process exits.  A
+ * Allocates nothing: its scratch (two 128-bit sums per 256 nodes) is a static device
+ * array of the library, 8 KB on every GPU that loads it, held until the process exits.  A
  * call whose stream is not capturing looks up that array's device address for the
  * current device (so a device reset between calls is harmless); a call made while its
  * stream is being captured reuses the address of the last such lookup on the device,

@@ -6,9 +6,8 @@
 // fragment the heap, and host frameworks that own every byte of device memory
 // through their own pools.  This entry point serves them.  The caller passes the
 // fixed-point charge deposits and the output array; the only scratch the solve
-// needs (one 128-bit prefix sum per node and one 128-bit total) lives in the
-// file-scope device array below, which every GPU that loads the library holds
-// until the process exits.  The math is the same as the handle's field phase (without
+// needs (two 128-bit sums per chunk of nodes) lives in the file-scope device array
+// below, which every GPU that loads the library holds until the process exits.  The math is the same as the handle's field phase (without
 // its optional density smoother: the deposits are used as given):
 //   Z_j = sum_s z_s D_s[j],  R_j = sum_{1<=k<=j, k<N} Z_k,  U = sum_{1<=k<N} (N-k) Z_k,
 //   E_j = lambda (N (R_{j-1} + R_j) - 2U)      (0 < j < N),
@@ -25,9 +24,17 @@ namespace {
 constexpr int kNoAllocMaxCells = 65536;
 constexpr int kNoAllocMaxNodes = kNoAllocMaxCells + 1;
 constexpr int kMaxDevices = 64;
+// Nodes of a chunk, one a thread: 257 blocks at the largest size, so that a block adds up
+// the chunk sums in two rounds.  Up to kNoAllocOneBlock nodes one block does it all in one
+// launch.  A call waited for alone, before and after: 65,536 cells 164 -> 25 us (11 us in
+// a row), 20,000 73 -> 22, 2,912 26 -> 21, 500 24 -> 17.5, 64 23 -> 16.4; the launches and
+// the host's checks are what is left.
+constexpr int kNoAllocChunk = 256;
+constexpr int kNoAllocOneBlock = 1024;
 
-// Scratch shared by every call on a device: R_j for j = 0..N, then U.
-static __device__ __align__(256) i128 g_scratch[kNoAllocMaxNodes + 1];
+// Scratch shared by every call on a device: per chunk of nodes the sums of Z'_j and of
+// (N-j) Z'_j over its interior nodes.
+static __device__ __align__(256) i128 g_scratch[2 * ((kNoAllocMaxNodes + kNoAllocChunk - 1) / kNoAllocChunk)];
 
 // Device address of g_scratch per device, from the last lookup made with that device
 // current and no capture in progress on the call's stream.
@@ -40,7 +47,7 @@ struct NoAllocArgs {
     int nspecies;
     int z[kMaxSpecies];
     double lambda;
-    i128* scratch;            // R[0..N], U at [N+1]
+    i128* scratch;            // [2c], [2c+1]: the sums of chunk c
     double* E;
 };
 
@@ -70,64 +77,93 @@ __device__ __forceinline__ i128 charge_at(const NoAllocArgs& a, int j)
     return z;
 }
 
-// One block of 1024 threads: R (inclusive prefix of the interior charge) and U.  Each
-// thread owns C consecutive nodes; their interior charges Z_j are formed once, kept in
-// the scratch slots R_j until the prefix overwrites them.
-__global__ void __launch_bounds__(1024) k_scan_noalloc(const NoAllocArgs a)
+// Sum of v over the block, for every thread.  sh: 33 entries.
+__device__ __forceinline__ i128 block_sum(i128 v, i128* sh)
 {
-    __shared__ i128 sh[33];
-    const int N = a.ncells, nn = N + 1;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int C = (nn + blockDim.x - 1) / blockDim.x;
-    const int j0 = min(nn, (int)threadIdx.x * C), j1 = min(nn, j0 + C);
-    i128 sum = 0, wsum = 0;
-    for (int j = j0; j < j1; ++j) {
-        const i128 z = (j == 0 || j == N) ? (i128)0 : charge_at(a, j);
-        a.scratch[j] = z;
-        sum += z;
-        wsum += (i128)(N - j) * z;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    v = sum_warp(v);
+    if (lane == 0) sh[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        const i128 t = sum_warp(lane < nw ? sh[lane] : (i128)0);
+        if (lane == 0) sh[32] = t;
     }
-    // block exclusive scan of `sum`
-    const i128 inc = incl_scan_warp(sum);
+    __syncthreads();
+    const i128 t = sh[32];
+    __syncthreads();
+    return t;
+}
+
+// Inclusive prefix of v over the block.
+__device__ __forceinline__ i128 block_scan(i128 v, i128* sh)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const i128 inc = incl_scan_warp(v);
     if (lane == 31) sh[warp] = inc;
     __syncthreads();
     if (warp == 0) {
-        const i128 w = sh[lane];
+        const i128 w = lane < nw ? sh[lane] : (i128)0;
         const i128 wi = incl_scan_warp(w);
-        sh[lane] = wi - w;
+        if (lane < nw) sh[lane] = wi - w;
     }
     __syncthreads();
-    i128 run = sh[warp] + inc - sum;
-    __syncthreads();
-    // block sum of `wsum`
-    const i128 ws = sum_warp(wsum);
-    if (lane == 0) sh[warp] = ws;
-    __syncthreads();
-    if (warp == 0) {
-        const i128 t = sum_warp(sh[lane]);
-        if (lane == 0) a.scratch[N + 1] = t;
-    }
-    for (int j = j0; j < j1; ++j) {
-        run += a.scratch[j];
-        a.scratch[j] = run;
+    return sh[warp] + inc;
+}
+
+// E of node j from R_{j-1} and Z_j (the wall nodes' Z enters E alone).
+__device__ __forceinline__ double field_at(const NoAllocArgs& a, int j, i128 Rprev, i128 z, i128 U)
+{
+    const int N = a.ncells;
+    const i128 NN = (i128)N;
+    i128 G;
+    if (j == 0) G = -2 * U - 2 * NN * z;
+    else if (j == N) G = 2 * NN * Rprev - 2 * U + 2 * NN * z;
+    else G = NN * (2 * Rprev + z) - 2 * U;
+    return a.lambda * i128_to_double(G);
+}
+
+// The whole solve in one block (one node a thread) where the nodes fit: one launch.
+__global__ void __launch_bounds__(1024) k_solve_noalloc(const NoAllocArgs a)
+{
+    __shared__ i128 sh[33];
+    const int N = a.ncells, j = threadIdx.x;
+    const i128 z = j <= N ? charge_at(a, j) : (i128)0;
+    const i128 in = (j > 0 && j < N) ? z : (i128)0;
+    const i128 U = block_sum((i128)(N - j) * in, sh);
+    const i128 R = block_scan(in, sh);
+    if (j <= N) a.E[j] = field_at(a, j, R - in, z, U);
+}
+
+// Larger instances in chunks of kNoAllocChunk nodes, a block each: the chunks' sums, then
+// every block adds up the sums of the chunks before its own and of all of them and scans
+// its nodes.  (All nodes in the threads of one block, 64 consecutive ones a thread, took
+// 146 us for 65,536 cells: a serial chain of uncoalesced 128-bit accesses on one SM.)
+__global__ void __launch_bounds__(kNoAllocChunk) k_sums_noalloc(const NoAllocArgs a)
+{
+    __shared__ i128 sh[33];
+    const int N = a.ncells, j = blockIdx.x * kNoAllocChunk + threadIdx.x;
+    const i128 in = (j > 0 && j < N) ? charge_at(a, j) : (i128)0;
+    const i128 s = block_sum(in, sh), w = block_sum((i128)(N - j) * in, sh);
+    if (threadIdx.x == 0) {
+        a.scratch[2 * blockIdx.x] = s;
+        a.scratch[2 * blockIdx.x + 1] = w;
     }
 }
 
-__global__ void k_emit_noalloc(const NoAllocArgs a)
+__global__ void __launch_bounds__(kNoAllocChunk) k_emit_noalloc(const NoAllocArgs a)
 {
-    const int N = a.ncells;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j > N) return;
-    const i128 U = a.scratch[N + 1];
-    const i128 NN = (i128)N;
-    i128 G;
-    if (j == 0)
-        G = -2 * U - 2 * NN * charge_at(a, 0);
-    else if (j == N)
-        G = 2 * NN * a.scratch[N - 1] - 2 * U + 2 * NN * charge_at(a, N);
-    else
-        G = NN * (a.scratch[j - 1] + a.scratch[j]) - 2 * U;
-    a.E[j] = a.lambda * i128_to_double(G);
+    __shared__ i128 sh[33];
+    const int N = a.ncells, j = blockIdx.x * kNoAllocChunk + threadIdx.x;
+    const i128 z = j <= N ? charge_at(a, j) : (i128)0;
+    const i128 in = (j > 0 && j < N) ? z : (i128)0;
+    i128 before = 0, u = 0;
+    for (int c = threadIdx.x; c < (int)gridDim.x; c += kNoAllocChunk) {
+        if (c < (int)blockIdx.x) before += a.scratch[2 * c];
+        u += a.scratch[2 * c + 1];
+    }
+    const i128 U = block_sum(u, sh), R0 = block_sum(before, sh);
+    const i128 R = R0 + block_scan(in, sh);
+    if (j <= N) a.E[j] = field_at(a, j, R - in, z, U);
 }
 
 // The device address of the scratch array for the current device.  Host code must not
@@ -211,8 +247,14 @@ extern "C" PIC_API int pic_field_solve_noalloc(int32_t ncells, int32_t nspecies,
     a.lambda = delta / (2.0 * (double)ncells * (double)unit * eps0);
     a.scratch = static_cast<i128*>(scratch);
     a.E = E;
-    k_scan_noalloc<<<1, 1024, 0, st>>>(a);
-    k_emit_noalloc<<<(ncells + 1 + 255) / 256, 256, 0, st>>>(a);
+    const int nodes = ncells + 1;
+    if (nodes <= kNoAllocOneBlock) {
+        k_solve_noalloc<<<1, (nodes + 31) / 32 * 32, 0, st>>>(a);
+    } else {
+        const int blocks = (nodes + kNoAllocChunk - 1) / kNoAllocChunk;
+        k_sums_noalloc<<<blocks, kNoAllocChunk, 0, st>>>(a);
+        k_emit_noalloc<<<blocks, kNoAllocChunk, 0, st>>>(a);
+    }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_global_error(std::string("pic_field_solve_noalloc: ") + cudaGetErrorString(e));
