@@ -43,6 +43,9 @@ namespace {
 
 thread_local std::string g_create_error;
 
+// Pinned memory of a handle for the diagnostics (larger packets are copied array by array).
+constexpr size_t kDiagPinned = (size_t)1 << 20;
+
 void mkdir_if_missing(const std::string& dir);
 
 struct Store {
@@ -127,7 +130,10 @@ struct pic_handle {
     int64_t ahead_tiles = 2;    // tiles per resident warp from which the mover fetches them ahead
     int64_t chunk_rounds = 200; // tiles per resident warp from which its warps take chunks of tiles
     std::vector<int> collide_nsteps;      // the distinct subcycling factors of colliding species
-    double *kin = nullptr, *phi_d = nullptr;
+    double* kin = nullptr;    // k_kinetic's block sums
+    char* diag = nullptr;     // the diagnostics' packet of one instance (pic_moments)
+    char* diag_h = nullptr;   // and its pinned copy: the head, and the arrays where they fit
+    size_t diag_h_bytes = 0;
     std::vector<void*> allocs;
     char* io = nullptr;       // staging of pic_load_particles / pic_get_particles host data
     size_t io_bytes = 0;
@@ -721,12 +727,9 @@ int do_sort(pic_handle* h)
     return PIC_OK;
 }
 
-// Synchronise and translate a latched device error.
-int sync_check(pic_handle* h)
+// Translate the device's status word.
+int latched(pic_handle* h, unsigned e)
 {
-    CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-    unsigned e = 0;
-    CUDA_TRY(h, cudaMemcpy(&e, h->err, sizeof(unsigned), cudaMemcpyDeviceToHost));
     if (e == 0) return PIC_OK;
     int code = PIC_ECUDA;
     std::string msg;
@@ -739,6 +742,15 @@ int sync_check(pic_handle* h)
     h->state = code;
     h->last_error = msg;
     return code;
+}
+
+// Synchronise and report a latched device error.
+int sync_check(pic_handle* h)
+{
+    CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    unsigned e = 0;
+    CUDA_TRY(h, cudaMemcpy(&e, h->err, sizeof(unsigned), cudaMemcpyDeviceToHost));
+    return latched(h, e);
 }
 
 int collect_times(pic_handle* h)
@@ -1152,7 +1164,14 @@ int pic_create(const pic_config* cfg, pic_handle** out)
     if (rc == PIC_OK && h->any_target) rc = dalloc(h, &h->tcount, (size_t)snode);
     if (rc == PIC_OK && h->any_target) rc = dalloc(h, &h->treq, (size_t)snode);
     if (rc == PIC_OK && h->any_target) rc = dalloc(h, &h->vlist, (size_t)std::max<int64_t>(ev, 1));
-    if (rc == PIC_OK) rc = dalloc(h, &h->phi_d, (size_t)h->max_nodes);
+    const size_t diag_bytes = sizeof(DiagHead) + (size_t)(PIC_MAX_SPECIES + 2) * h->max_nodes * 8;
+    if (rc == PIC_OK) rc = dalloc(h, &h->diag, diag_bytes);
+    h->diag_h_bytes = std::min<size_t>(diag_bytes, kDiagPinned);
+    if (rc == PIC_OK && cudaMallocHost((void**)&h->diag_h, h->diag_h_bytes) != cudaSuccess) {
+        cudaGetLastError();
+        h->diag_h = nullptr;
+        rc = fail(h, PIC_ENOMEM, "cudaMallocHost of the diagnostics' buffer failed");
+    }
     if (rc == PIC_OK) rc = dalloc(h, &h->segd, (size_t)h->nseg);
     if (rc == PIC_OK) rc = dalloc(h, &h->instd, (size_t)h->ninst);
     if (rc == PIC_OK) rc = dalloc(h, &h->newn, (size_t)h->nseg);
@@ -1175,7 +1194,7 @@ int pic_create(const pic_config* cfg, pic_handle** out)
     if (rc == PIC_OK) rc = dalloc(h, &h->cell_part, (size_t)h->nseg * h->cell_chunks);
     if (rc == PIC_OK) rc = dalloc(h, &h->err, 1);
     if (rc == PIC_OK) rc = dalloc(h, &h->step_d, 2);
-    if (rc == PIC_OK) rc = dalloc(h, &h->kin, (size_t)PIC_MAX_SPECIES);
+    if (rc == PIC_OK) rc = dalloc(h, &h->kin, (size_t)PIC_MAX_SPECIES * kKineticBlocks);
     if (rc) return bail(rc);
 
     cudaStream_t s = h->stream;
@@ -1618,66 +1637,72 @@ int pic_moments(pic_handle* h, int32_t inst, pic_moments_out* out, double* densi
     const InstParams& ip = h->insth[inst];
     const int ns = I.nspecies, N = I.ncells;
     cudaStream_t s = h->stream;
-    CUDA_TRY(h, cudaMemsetAsync(h->kin, 0, sizeof(double) * PIC_MAX_SPECIES, s));
     const Store& S = h->st[h->cur];
     int64_t maxslots = 0;
     for (int k = 0; k < ns; ++k) maxslots = std::max(maxslots, h->segh[ip.seg0 + k].cap);
-    CUDA_TRY(h, launch_kinetic(h->segd, ip.seg0, ns, maxslots, S.cell, S.ux, S.uy, S.uz,
+    CUDA_TRY(h, launch_kinetic(h->segd, h->seg_n, ip.seg0, ns, maxslots, S.cell, S.ux, S.uy, S.uz,
                                h->precision, h->kin, s));
-    if (phi && I.field == PIC_FIELD_POISSON)
-        CUDA_TRY(h, launch_potential(field_args(h), inst, I.dx, h->phi_d, s));
-    if ((rc = sync_check(h))) return rc;
-
+    // one packet: the head, then the arrays asked for, copied to the host in one piece and
+    // waited for once (twelve blocking copies and the conversions on the host took some
+    // 150 us a call)
+    const bool poisson = I.field == PIC_FIELD_POISSON;
+    const size_t nodes = (size_t)(N + 1) * 8;
+    size_t bytes = sizeof(DiagHead);
+    auto take = [&](bool on, size_t n) {
+        char* p = on ? h->diag + bytes : nullptr;
+        if (on) bytes += n;
+        return reinterpret_cast<double*>(p);
+    };
+    DiagArgs d;
+    d.inst = inst;
+    d.head = reinterpret_cast<DiagHead*>(h->diag);
+    d.density = take(density != nullptr, nodes * ns);
+    d.phi = take(phi && poisson, nodes);
+    d.E = take(E != nullptr, nodes);
+    for (int k = 0; k < ns; ++k) d.wdx[k] = I.sp[k].weight / I.dx;
+    d.unit = h->precision == PIC_FP64 ? 281474976710656.0 : 16777216.0;
+    d.dx = I.dx;
+    d.periodic = I.bc == PIC_BC_PERIODIC ? 1 : 0;
+    d.kin = h->kin;
+    d.kin_blocks = kinetic_blocks(maxslots);
+    d.seg_live = h->seg_live;
+    d.wall_count = h->wall_count;
+    d.wall_energy = h->wall_energy;
+    d.collisions = h->collisions;
+    d.next_id = h->next_id;
+    d.err = h->err;
+    CUDA_TRY(h, launch_diag(field_args(h), d, ip.nchunk, s));
+    const bool whole = bytes <= h->diag_h_bytes;
+    CUDA_TRY(h, cudaMemcpyAsync(h->diag_h, h->diag, whole ? bytes : sizeof(DiagHead),
+                                cudaMemcpyDeviceToHost, s));
+    CUDA_TRY(h, cudaStreamSynchronize(s));
+    const DiagHead& head = *reinterpret_cast<const DiagHead*>(h->diag_h);
+    if ((rc = latched(h, (unsigned)head.err))) return rc;
+    auto give = [&](double* to, const double* from, size_t n) -> cudaError_t {
+        if (!to || !from) return cudaSuccess;
+        const char* src = reinterpret_cast<const char*>(from);
+        if (!whole) return cudaMemcpy(to, src, n, cudaMemcpyDeviceToHost);
+        std::memcpy(to, h->diag_h + (src - h->diag), n);
+        return cudaSuccess;
+    };
+    CUDA_TRY(h, give(density, d.density, nodes * ns));
+    CUDA_TRY(h, give(phi, d.phi, nodes));
+    CUDA_TRY(h, give(E, d.E, nodes));
     std::memset(out, 0, sizeof(*out));
-    int64_t step = 0;
-    std::vector<unsigned long long> live(ns), wc(2 * ns), col(kMaxProc);
-    std::vector<double> we(2 * ns), kin(ns);
-    CUDA_TRY(h, cudaMemcpy(&step, h->step_d + 1, 8, cudaMemcpyDeviceToHost));
-    CUDA_TRY(h, cudaMemcpy(live.data(), h->seg_live + ip.seg0, 8 * ns, cudaMemcpyDeviceToHost));
-    CUDA_TRY(h, cudaMemcpy(wc.data(), h->wall_count + 2 * ip.seg0, 16 * ns, cudaMemcpyDeviceToHost));
-    CUDA_TRY(h, cudaMemcpy(we.data(), h->wall_energy + 2 * ip.seg0, 16 * ns, cudaMemcpyDeviceToHost));
-    CUDA_TRY(h, cudaMemcpy(col.data(), h->collisions + (size_t)inst * kMaxProc, 8 * kMaxProc, cudaMemcpyDeviceToHost));
-    CUDA_TRY(h, cudaMemcpy(kin.data(), h->kin, 8 * ns, cudaMemcpyDeviceToHost));
-    unsigned long long nid = 0;
-    CUDA_TRY(h, cudaMemcpy(&nid, h->next_id + inst, 8, cudaMemcpyDeviceToHost));
-    out->step = step;
-    out->next_id = (int64_t)nid;
+    out->step = head.step;
+    out->next_id = (int64_t)head.next_id;
     for (int k = 0; k < ns; ++k) {
-        out->live[k] = (int64_t)live[k];
-        out->wall_count[k][0] = (int64_t)wc[2 * k];
-        out->wall_count[k][1] = (int64_t)wc[2 * k + 1];
-        out->wall_energy[k][0] = we[2 * k];
-        out->wall_energy[k][1] = we[2 * k + 1];
-        out->kinetic[k] = kin[k];
-    }
-    for (int q = 0; q < I.nproc; ++q) out->collisions[q] = (int64_t)col[q];
-    if (density) {
-        const double Sunit = h->precision == PIC_FP64 ? 281474976710656.0 : 16777216.0;
-        std::vector<unsigned long long> d((size_t)(N + 1));
-        for (int k = 0; k < ns; ++k) {
-            const SegParams& P = h->segh[ip.seg0 + k];
-            CUDA_TRY(h, cudaMemcpy(d.data(), h->dep_last + P.node, 8 * (size_t)(N + 1), cudaMemcpyDeviceToHost));
-            const double wdx = I.sp[k].weight / I.dx;
-            double* o = density + (size_t)k * (N + 1);
-            for (int j = 0; j <= N; ++j) o[j] = wdx * ((double)d[j] / Sunit);
-            if (I.bc == PIC_BC_PERIODIC) {
-                const double v = wdx * ((double)(d[0] + d[N]) / Sunit);
-                o[0] = v;
-                o[N] = v;
-            } else {
-                o[0] *= 2.0;
-                o[N] *= 2.0;
-            }
+        out->live[k] = (int64_t)head.live[k];
+        for (int w = 0; w < 2; ++w) {
+            out->wall_count[k][w] = (int64_t)head.wall_count[2 * k + w];
+            out->wall_energy[k][w] = head.wall_energy[2 * k + w];
         }
+        out->kinetic[k] = head.kinetic[k];
     }
-    if (E) CUDA_TRY(h, cudaMemcpy(E, h->E + ip.inode, 8 * (size_t)(N + 1), cudaMemcpyDeviceToHost));
-    if (phi) {
-        if (I.field == PIC_FIELD_POISSON) {
-            CUDA_TRY(h, cudaMemcpy(phi, h->phi_d, 8 * (size_t)(N + 1), cudaMemcpyDeviceToHost));
-        } else {
-            const double e0 = I.field == PIC_FIELD_EXTERNAL ? I.E_ext : 0.0;
-            for (int j = 0; j <= N; ++j) phi[j] = -e0 * ((double)j * I.dx);
-        }
+    for (int q = 0; q < I.nproc; ++q) out->collisions[q] = (int64_t)head.collisions[q];
+    if (phi && !poisson) {
+        const double e0 = I.field == PIC_FIELD_EXTERNAL ? I.E_ext : 0.0;
+        for (int j = 0; j <= N; ++j) phi[j] = -e0 * ((double)j * I.dx);
     }
     return PIC_OK;
 }
@@ -1947,6 +1972,7 @@ int pic_destroy(pic_handle* h)
     drop_graphs(h);
     for (void* p : h->allocs) cudaFree(p);
     if (h->io) cudaFree(h->io);
+    if (h->diag_h) cudaFreeHost(h->diag_h);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
     if (h->side_stream) cudaStreamDestroy(h->side_stream);

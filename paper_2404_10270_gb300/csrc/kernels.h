@@ -57,9 +57,38 @@ struct FieldArgs {
     int any_poisson;
 };
 cudaError_t launch_field(const FieldArgs& f, bool advance_step, cudaStream_t st);
-// potential of instance `inst` (FIELD_POISSON) into phi[0..N]
-cudaError_t launch_potential(const FieldArgs& f, int inst, double dx, double* phi,
-                             cudaStream_t st);
+// The diagnostics of one instance: a packet of a head and (where the pointers are not null)
+// node arrays, written by one launch after launch_kinetic.
+struct DiagHead {
+    int64_t step;
+    unsigned long long next_id;
+    unsigned long long live[kMaxSpecies];
+    unsigned long long wall_count[2 * kMaxSpecies];
+    double wall_energy[2 * kMaxSpecies];
+    unsigned long long collisions[kMaxProc];
+    double kinetic[kMaxSpecies];
+    unsigned long long err;  // the status word
+};
+struct DiagArgs {
+    int inst;
+    DiagHead* head;
+    double* density;        // nspecies x (ncells+1), or null
+    double* phi;            // ncells+1, or null (also where there is no Poisson solve)
+    double* E;              // ncells+1, or null
+    double wdx[kMaxSpecies];  // weight / dx
+    double unit;            // of the fixed-point deposit
+    double dx;
+    int periodic;
+    const double* kin;      // k_kinetic's block sums, [species][kin_blocks]
+    int kin_blocks;
+    const unsigned long long* seg_live;
+    const unsigned long long* wall_count;
+    const double* wall_energy;
+    const unsigned long long* collisions;
+    const unsigned long long* next_id;
+    const unsigned* err;
+};
+cudaError_t launch_diag(const FieldArgs& f, const DiagArgs& d, int nchunk, cudaStream_t st);
 
 // Snapshot each segment's slot count, rounded up to a whole quad, as the count to
 // move, and build the tile prefix (tiles of `tile_quads` quads).
@@ -183,9 +212,12 @@ cudaError_t launch_get_write(GetArgs g, int64_t block0, int64_t nblocks, cudaStr
 cudaError_t launch_set_yp(void* s_yp, int64_t base, const double* in, int64_t n, int precision,
                           cudaStream_t st);
 
-// sum of kefac |u|^2 over live particles of segments [s0, s0+ns) into out[ns]
-cudaError_t launch_kinetic(const SegParams* seg, int s0, int ns, int64_t max_slots,
-                           const int32_t* cell, const void* ux, const void* uy,
+// sums of |u|^2 over the live particles of segments [s0, s0+ns), one per block:
+// out[ns][kinetic_blocks(max_slots)]
+constexpr int kKineticBlocks = 152 * 8;
+int kinetic_blocks(int64_t max_slots);
+cudaError_t launch_kinetic(const SegParams* seg, const unsigned long long* seg_n, int s0, int ns,
+                           int64_t max_slots, const int32_t* cell, const void* ux, const void* uy,
                            const void* uz, int precision, double* out, cudaStream_t st);
 
 cudaError_t launch_philox(uint64_t key, const uint32_t* ctr, uint32_t* out, int64_t n,
