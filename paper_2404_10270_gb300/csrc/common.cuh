@@ -79,7 +79,8 @@ struct SegParams {
     int64_t node;          // first entry of this segment's node arrays
     int64_t inode;         // first entry of the instance's node arrays (E)
     uint32_t key0, key1;   // Philox key = instance seed
-    double accel;          // c_s = (q/m) dt^2/dx: A = c_s E in cells/step^2
+    double accel;          // c_s = (q/m) dt^2/dx: A = c_s E in cells/step^2 (half of it in a
+                           // magnetized instance, whose push adds it twice)
     double t[3], s[3];     // Boris: t = (q/m) B dt/2, s = 2t/(1+t.t)
     float tf[3], sf[3];    // the same rounded to float (the FP32 form's values)
     double kefac;          // w m (dx/dt)^2 / 2: energy of |u|^2 = 1 (cells/step)^2
@@ -99,7 +100,7 @@ struct SegParams {
     int32_t is_target;     // the instance's neutral particle target
     int32_t mag;           // the instance has a magnetic field (Boris push)
     int32_t sn2d;          // the species also drifts in y (Listing 1: yp += nstep*vy)
-    int32_t pad;
+    int32_t planar;        // t[2] = s[2] = 0: B lies in the x-y plane (either form's values)
 };
 
 // Whether a species with subcycling moves on step n (counted from 0).  On the steps it

@@ -377,6 +377,8 @@ void seg_constants(const pic_instance& I, int s, SegParams* P)
     const double vs = dt / I.dx;
     const double qm = S.charge / S.mass;
     P->accel = qm * (dt * dt / I.dx);
+    // the Boris push adds half of it twice (exact: a power of two)
+    if (I.B[0] != 0.0 || I.B[1] != 0.0 || I.B[2] != 0.0) P->accel *= 0.5;
     const double qmh = qm * (0.5 * dt);
     for (int k = 0; k < 3; ++k) P->t[k] = qmh * I.B[k];
     const double tt = P->t[0] * P->t[0] + P->t[1] * P->t[1] + P->t[2] * P->t[2];
@@ -386,6 +388,7 @@ void seg_constants(const pic_instance& I, int s, SegParams* P)
         P->tf[k] = (float)P->t[k];
         P->sf[k] = (float)P->s[k];
     }
+    P->planar = P->t[2] == 0.0 && P->s[2] == 0.0 ? 1 : 0;
     const double dxdt = I.dx / dt;
     P->kefac = 0.5 * S.mass * S.weight * (dxdt * dxdt);
     P->vinj = std::sqrt(S.temperature / S.mass) * vs;
