@@ -1899,7 +1899,7 @@ int pic_restore_counters(pic_handle* h, int64_t step, const uint64_t* next_id)
     const int64_t both[2] = {step, step};
     CUDA_TRY(h, cudaMemcpy(h->step_d, both, 16, cudaMemcpyHostToDevice));
     if (step != h->step_h) {
-        CUDA_TRY(h, launch_rebase_clocks(h->segd, h->nseg, h->st[h->cur].cell, h->step_h, step, h->stream));
+        CUDA_TRY(h, launch_rebase_clocks(h->segd, h->seg_n, h->nseg, h->max_cap, h->st[h->cur].cell, h->step_h, step, h->stream));
         CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     }
     if (next_id) {

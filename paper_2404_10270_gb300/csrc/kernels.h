@@ -173,8 +173,9 @@ struct LoadArgs {
 cudaError_t launch_load(const LoadArgs& l, cudaStream_t st);
 // clocks kept at their distance from each species' next moving step when the step
 // counter is set from `from` to `to`
-cudaError_t launch_rebase_clocks(const SegParams* seg, int nseg, int32_t* cell, int64_t from,
-                                 int64_t to, cudaStream_t st);
+cudaError_t launch_rebase_clocks(const SegParams* seg, const unsigned long long* seg_n, int nseg,
+                                 int64_t max_slots, int32_t* cell, int64_t from, int64_t to,
+                                 cudaStream_t st);
 
 struct GetArgs {
     const int32_t* s_cell;
