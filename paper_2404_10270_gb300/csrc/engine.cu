@@ -2,8 +2,6 @@
 // layout, the per-step launch sequence and the synchronising queries.
 //
 // Launch sequence of one time step (all on the handle's stream):
-//   k_tiles     snapshot each segment's slot count (rounded to a whole quad), build the
-//               tile list, empty the rare-event queue
 //   k_move      gather, push, move, periodic wrap, collision clock, fixed-point deposit;
 //               walls and collision candidates are queued (mover.cuh); a large batch takes
 //               another variant on the steps on which every clock tests
@@ -12,7 +10,8 @@
 //   k_victims   neutral particle targets: the ionized targets become ions (events.cuh)
 //   k_births    number this step's ionization products (only with ionization)
 //   k_field     exact integer Poisson solve (optional smoother) -> E -> node pairs of
-//               pre-scaled accelerations, and hand-over of the deposit (field.cu)
+//               pre-scaled accelerations, hand-over of the deposit, and the next step's
+//               tile list (each segment's slot count, rounded to a whole quad) (field.cu)
 //   the sort, every `sort_interval` steps: the step before counts the particles per cell
 //   at its end (k_move's deposit, k_events); the sort step scans the counts
 //   (k_cell_partial, k_cell_scan), its mover writes every particle into its cell-ordered
@@ -121,9 +120,9 @@ struct pic_handle {
     unsigned long long* rare_count = nullptr;
     int grid_events = 0;
     unsigned* err = nullptr;
-    // the step count: [0] the step the kernels of a step read (set from [1] by k_tiles,
-    // the first kernel of every step), [1] the steps completed (the field phase of a
-    // step writes [0] + 1), so that the field phase may run beside the event kernels
+    // the step count: [1] the steps completed (the mover reads it; the field phase of a step
+    // writes [0] + 1), [0] the step under way (the mover copies it from [1] for the kernels
+    // after it), so that the field phase may run beside the event kernels
     int64_t* step_d = nullptr;
     bool test_all = true;  // every clock may need a test in the next step (after a load)
     int64_t full_min = (int64_t)1 << 24;  // particle slots from which test steps take the kFull mover
@@ -527,6 +526,17 @@ SortArgs sort_args(pic_handle* h)
     return a;
 }
 
+TileArgs tile_args(pic_handle* h)
+{
+    TileArgs t;
+    t.seg_n = h->seg_n;
+    t.seg_nmove = h->seg_nmove;
+    t.tile_start = h->tile_start;
+    t.nseg = h->nseg;
+    t.tile_quads = 32;
+    return t;
+}
+
 FieldArgs field_args(pic_handle* h)
 {
     FieldArgs f;
@@ -548,6 +558,9 @@ FieldArgs field_args(pic_handle* h)
     f.step = h->step_d;
     f.any_poisson = h->any_poisson ? 1 : 0;
     f.zs = h->zs;
+    f.tiles = tile_args(h);
+    // (the y drift on the second stream still reads this step's list)
+    if (h->any_sn2d) f.tiles.nseg = 0;
     return f;
 }
 
@@ -683,8 +696,7 @@ int launch_tiles_h(pic_handle* h)
 {
     Span sp(h, 3);
     h->kernels += 1;
-    CUDA_TRY(h, launch_tiles(h->segd, h->seg_n, h->seg_nmove, h->tile_start, h->nseg, 32,
-                             h->rare_count, h->step_d, h->stream));
+    CUDA_TRY(h, launch_tiles(h->segd, tile_args(h), h->stream));
     return PIC_OK;
 }
 
@@ -707,8 +719,9 @@ int ensure_fields(pic_handle* h)
     if ((rc = launch_move(h, false))) return rc;
     {
         Span sp(h, 1);
-        h->kernels += h->any_poisson ? 2 : 1;
-        CUDA_TRY(h, launch_field(field_args(h), false, h->stream));
+        const FieldArgs f = field_args(h);
+        h->kernels += field_launches(f);
+        CUDA_TRY(h, launch_field(f, false, h->stream));
     }
     h->stale = false;
     return PIC_OK;
@@ -720,14 +733,16 @@ int do_sort(pic_handle* h)
 {
     int rc = launch_tiles_h(h);
     if (rc) return rc;
-    Span sp(h, 2);
-    CUDA_TRY(h, cudaMemsetAsync(h->hist, 0, sizeof(unsigned) * (size_t)h->seg_nodes, h->stream));
     const SortArgs a = sort_args(h);
     h->hist_ready = false;
-    h->kernels += h->any_target ? 6 : 5;
-    CUDA_TRY(h, launch_sort(a, h->nt, h->sms, h->stream));
+    {
+        Span sp(h, 2);
+        CUDA_TRY(h, cudaMemsetAsync(h->hist, 0, sizeof(unsigned) * (size_t)h->seg_nodes, h->stream));
+        h->kernels += h->any_target ? 6 : 5;
+        CUDA_TRY(h, launch_sort(a, h->nt, h->sms, h->stream));
+    }
     h->cur = 1 - h->cur;
-    return PIC_OK;
+    return launch_tiles_h(h);  // the new counts' tiles
 }
 
 // Translate the device's status word.
@@ -1126,7 +1141,8 @@ int pic_create(const pic_config* cfg, pic_handle** out)
         return bail(PIC_ECUDA);
     }
     h->sms = prop.multiProcessorCount;
-    h->grid_events = (int)std::min<int64_t>((h->rare_cap + 127) / 128, (int64_t)16 * h->sms);
+    h->grid_events = (int)std::min<int64_t>((h->rare_cap - 65536 + 127) / 128, (int64_t)4 * h->sms);
+    h->grid_events = std::max(h->grid_events, std::min(h->sms, 32));
     // one warp per requested target cell: at most the ionization events of a step
     h->grid_victims = (int)std::min<int64_t>((std::max<int64_t>(h->ev_total, 1) + 3) / 4, (int64_t)4 * h->sms);
     std::snprintf(h->gpu_name, sizeof(h->gpu_name), "%s", prop.name);
@@ -1189,7 +1205,7 @@ int pic_create(const pic_config* cfg, pic_handle** out)
     if (rc == PIC_OK) rc = dalloc(h, &h->events, (size_t)std::max<int64_t>(ev, 1));
     if (rc == PIC_OK) rc = dalloc(h, &h->ev_count, (size_t)h->ninst);
     if (rc == PIC_OK) rc = dalloc(h, &h->rare, (size_t)h->rare_cap);
-    if (rc == PIC_OK) rc = dalloc(h, &h->rare_count, 2);
+    if (rc == PIC_OK) rc = dalloc(h, &h->rare_count, 4);
     if (rc == PIC_OK) rc = dalloc(h, &h->next_id, (size_t)h->ninst);
     if (rc == PIC_OK) rc = dalloc(h, &h->birth_keys_a, (size_t)std::max<int64_t>(h->ev_total, 1));
     if (rc == PIC_OK) rc = dalloc(h, &h->birth_keys_b, (size_t)std::max<int64_t>(h->ev_total, 1));
@@ -1213,7 +1229,7 @@ int pic_create(const pic_config* cfg, pic_handle** out)
         if (e == cudaSuccess) e = launch_fill_i32(h->st[b].cell, 0, slot, -1, s);
     }
     if (e == cudaSuccess) e = z(h->accel, (size_t)snode * 2 * T);
-    if (e == cudaSuccess) e = z(h->rare_count, 16);
+    if (e == cudaSuccess) e = z(h->rare_count, 32);
     if (e == cudaSuccess) e = z(h->dep, (size_t)snode * 8);
     if (e == cudaSuccess) e = z(h->dep_last, (size_t)snode * 8);
     if (e == cudaSuccess && h->any_target) e = z(h->tcount, (size_t)snode * 4);
@@ -1434,7 +1450,9 @@ int enqueue_step(pic_handle* h)
     } else if (fold && (h->step_h + 2) % K == 0) {
         phase = kCount;
     }
-    if ((rc = launch_tiles_h(h))) return rc;
+    // (the tile list comes from the field phase of the step before, the initial one or the
+    // separate sort)
+    if (h->any_sn2d && (rc = launch_tiles_h(h))) return rc;
     if ((rc = launch_move(h, true, phase))) return rc;
     h->hist_ready = phase == kCount;
     // Work that shares no word with the rest of the step runs on the side stream, forked
@@ -1469,8 +1487,9 @@ int enqueue_step(pic_handle* h)
     }
     {
         Span sp(h, 1);
-        h->kernels += h->any_poisson ? 2 : 1;
-        CUDA_TRY(h, launch_field(field_args(h), true, h->stream));
+        const FieldArgs f = field_args(h);
+        h->kernels += field_launches(f);
+        CUDA_TRY(h, launch_field(f, true, h->stream));
     }
     if (joined) CUDA_TRY(h, cudaStreamWaitEvent(h->stream, h->ev_join, 0));
     h->step_h += 1;

@@ -247,9 +247,25 @@ __device__ __forceinline__ void count_by_key(unsigned long long* counts, int key
         atomicAdd(counts + key, (unsigned long long)__popc(grp));
 }
 
-// One thread per queued particle.  The loop is uniform across each warp (every lane
+// Empty the list that `count` counts once the last block of the kernel is done with it.
+__device__ __forceinline__ void empty_after_last(unsigned long long* count, unsigned long long* done)
+{
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicAdd(done, 1ull) + 1ull == gridDim.x) {
+        *count = 0ull;
+        *done = 0ull;
+    }
+}
+
+// One lane per queued particle.  The loop is uniform across each warp (every lane
 // takes the same iterations), so that the collision and wall counts can be combined
-// per warp before they reach memory.
+// per warp before they reach memory.  A step's few events go to as many SMs as they can
+// (consecutive groups to consecutive blocks, and fewer than 32 to a warp while there are
+// fewer than 32 per SM): the kernel waits for memory and, in the FP64 form, for a chain of
+// operations of which one warp alone fills an SM's FP64 pipe for 16 cycles each.
+constexpr unsigned kEventSpread = 152;  // SMs
 template <typename T>
 __global__ void __launch_bounds__(128) k_events(const __grid_constant__ MoveArgs a)
 {
@@ -260,12 +276,13 @@ __global__ void __launch_bounds__(128) k_events(const __grid_constant__ MoveArgs
     T* const uyp = static_cast<T*>(a.uy);
     T* const uzp = static_cast<T*>(a.uz);
     const unsigned long long lane = threadIdx.x & 31;
-    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-    for (unsigned long long w = (unsigned long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
+    const unsigned long long per = min(32ull, (n + kEventSpread - 1) / kEventSpread);
+    const unsigned long long stride = (unsigned long long)gridDim.x * (blockDim.x >> 5) * per;
+    for (unsigned long long w = ((unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * per;
          w < n; w += stride) {
         const unsigned long long i = w + lane;
         int ckey = -1, wkey = -1;  // collision counter, wall counter
-        bool ok = i < n;
+        bool ok = lane < per && i < n;
         uint64_t e = 0;
         if (ok) {
             e = a.rare[i];
@@ -318,6 +335,7 @@ __global__ void __launch_bounds__(128) k_events(const __grid_constant__ MoveArgs
         count_by_key(a.collisions, ckey);
         count_by_key(a.wall_count, wkey);
     }
+    empty_after_last(a.rare_count, a.rare_count + 2);
 }
 
 // Ionization against a neutral particle target: the r_j ionizations of cell j this step
@@ -439,6 +457,7 @@ __global__ void __launch_bounds__(128) k_victims(const __grid_constant__ MoveArg
             }
         }
     }
+    empty_after_last(a.rare_count + 1, a.rare_count + 3);
 }
 
 // The y drift of 2-D species (Listing 1: yp += nstep*vy), after the mover and before

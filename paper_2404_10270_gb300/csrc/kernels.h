@@ -33,6 +33,15 @@ int move_blocks_per_sm_f32(bool mag, bool sub, bool sort, bool yp, MoveMode mode
 int move_blocks_per_sm_f64(bool mag, bool sub, bool sort, bool yp, MoveMode mode, int nt);
 
 // ---- field phase and bookkeeping (field.cu) -------------------------------------
+// The tile list of a step: the slots of each segment to move, and the prefix of tiles of
+// `tile_quads` quads over all segments.  nseg = 0: none is built.
+struct TileArgs {
+    unsigned long long* seg_n;
+    int64_t* seg_nmove;
+    int64_t* tile_start;
+    int nseg;
+    int tile_quads;
+};
 struct FieldArgs {
     const SegParams* seg;
     const InstParams* inst;
@@ -55,7 +64,9 @@ struct FieldArgs {
     i128* zs;                         // per instance node arrays: 4x the smoothed node
                                       // charge (instances with the smoother), else unused
     int any_poisson;
+    TileArgs tiles;                   // the next step's tile list, built beside the field
 };
+int field_launches(const FieldArgs& f);  // kernels of a launch_field
 cudaError_t launch_field(const FieldArgs& f, bool advance_step, cudaStream_t st);
 // The diagnostics of one instance: a packet of a head and (where the pointers are not null)
 // node arrays, written by one launch after launch_kinetic.
@@ -90,13 +101,7 @@ struct DiagArgs {
 };
 cudaError_t launch_diag(const FieldArgs& f, const DiagArgs& d, int nchunk, cudaStream_t st);
 
-// Snapshot each segment's slot count, rounded up to a whole quad, as the count to
-// move, and build the tile prefix (tiles of `tile_quads` quads).
-// Also empties the rare-event queue and the target request list of the coming step
-// (rare_count[0] and [1]) and sets the step its kernels read: step[0] = step[1].
-cudaError_t launch_tiles(const SegParams* seg, unsigned long long* seg_n, int64_t* seg_nmove,
-                         int64_t* tile_start, int nseg, int tile_quads,
-                         unsigned long long* rare_count, int64_t* step, cudaStream_t st);
+cudaError_t launch_tiles(const SegParams* seg, const TileArgs& t, cudaStream_t st);
 
 // Number this step's ionization products by the rank of their parent id.
 // `done`: one zeroed counter per instance (left zeroed).

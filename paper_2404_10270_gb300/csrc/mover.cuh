@@ -85,9 +85,11 @@ struct MoveArgs {
     Event* events;
     unsigned long long* ev_count;       // [ninst]
     unsigned* err;
-    const int64_t* step;
+    int64_t* step;                      // [1] steps completed, [0] the step under way
     uint64_t* rare;                     // queue of rare events of this step (rare_pack)
-    unsigned long long* rare_count;     // [0]: entries queued this step, [1]: entries of vlist
+    // [0]: entries queued this step, [1]: entries of vlist, each emptied by the kernel that
+    // works through it, whose finished blocks [2] and [3] count
+    unsigned long long* rare_count;
     int64_t rare_cap;                   // queue entries
     // neutral particle targets (segment node arrays of the target segments): live
     // targets per cell as of the start of the step, ionization requests of the step,
@@ -892,7 +894,9 @@ k_move(const __grid_constant__ MoveArgs a)
     T* const uxp = static_cast<T*>(a.ux);
     T* const uyp = static_cast<T*>(a.uy);
     T* const uzp = static_cast<T*>(a.uz);
-    const int64_t step = MOVE ? *a.step : 0;
+    const int64_t step = MOVE ? a.step[1] : 0;
+    // the step under way, for the kernels after the mover
+    if (MOVE && blockIdx.x == 0 && threadIdx.x == 0) a.step[0] = step;
     // the warps' deposit windows and (FP64) scratch of add_crossed
     __shared__ __align__(16) uint32_t s_dwin[NT / 32][DepWin<Q>::words + CrossScratch<T>::words];
     uint32_t* const dwin = s_dwin[threadIdx.x >> 5];
@@ -1147,7 +1151,8 @@ k_move_sort(const __grid_constant__ MoveArgs a)
     T* const uxp = static_cast<T*>(a.ux);
     T* const uyp = static_cast<T*>(a.uy);
     T* const uzp = static_cast<T*>(a.uz);
-    const int64_t step = *a.step;
+    const int64_t step = a.step[1];
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.step[0] = step;
     const int64_t total = a.tile_start[a.nseg];
     int s = 0;
     int64_t s_begin = 0, s_end = -1;
