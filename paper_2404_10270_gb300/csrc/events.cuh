@@ -55,6 +55,10 @@ __device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, T* z0, T* z
     *z1 = r * s;
 }
 
+// What a warp of k_events does with its events: all of it, or one of four parts: walls and
+// the candidates' clocks; elastic and exciting collisions; charge exchange; ionization.
+enum : int { kRoleAll = -1, kRoleWall = 0, kRoleScatter = 1, kRoleCx = 2, kRoleIonize = 3 };
+
 // A null-collision candidate of one particle (velocity u in cells/step, after the
 // move): with a neutral particle target, first the target density (kept with
 // probability min(1, n_j / nref) by the word `wdens`), then the process slot from the
@@ -62,9 +66,10 @@ __device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, T* z0, T* z
 // kinematics.  Returns the instance-level index of the process that took place (u
 // changed), or -1 for a null event.  Ionization appends two particles (the electron
 // only with a particle target: the target particle itself becomes the ion, see
-// k_victims).  The caller counts the collision.
+// k_victims).  The caller counts the collision.  `role` (kRoleAll, or one of k_events'):
+// only the processes of that role take place, the others are another warp's.
 template <typename T>
-__device__ __forceinline__ int collide(const MoveArgs& a, const SegParams& P, int s,
+__device__ __forceinline__ int collide(int role, const MoveArgs& a, const SegParams& P, int s,
                                     uint32_t id, int64_t step, int j, T f, T& ux, T& uy,
                                     T& uz, uint32_t wsel, uint32_t wdens, int64_t pslot)
 {
@@ -81,6 +86,9 @@ __device__ __forceinline__ int collide(const MoveArgs& a, const SegParams& P, in
     const T u2 = ux * ux + uy * uy + uz * uz;
     if (!(u2 >= (T)P.thr_u2[q])) return -1;  // below threshold: null event
     const int kind = P.kind[q];
+    if (role != kRoleAll &&
+        role != (kind == PIC_PROC_CX ? kRoleCx : kind == PIC_PROC_IONIZE ? kRoleIonize : kRoleScatter))
+        return -1;
     if (kind == PIC_PROC_ELASTIC) {
         const uint4 r = draw(id, step, kRngScatter, P.key0, P.key1);
         T n[3];
@@ -263,8 +271,11 @@ __device__ __forceinline__ void empty_after_last(unsigned long long* count, unsi
 // takes the same iterations), so that the collision and wall counts can be combined
 // per warp before they reach memory.  A step's few events go to as many SMs as they can
 // (consecutive groups to consecutive blocks, and fewer than 32 to a warp while there are
-// fewer than 32 per SM): the kernel waits for memory and, in the FP64 form, for a chain of
-// operations of which one warp alone fills an SM's FP64 pipe for 16 cycles each.
+// fewer than 32 per SM), and each group is worked through by four warps that take one kind
+// of event each (kRole*): the kernel waits for memory and, in the FP64 form, for chains of
+// dependent FP64 operations (some 900 for a warp that has every kind, at 64 cycles each
+// whatever its number of lanes).  4,096 cells x 200 x 2 with source and ionization, FP64:
+// 33 -> 19 us; 256 cells FP64 with walls, elastic and charge exchange: 13.1 -> 11.9.
 constexpr unsigned kEventSpread = 152;  // SMs
 template <typename T>
 __global__ void __launch_bounds__(128) k_events(const __grid_constant__ MoveArgs a)
@@ -277,9 +288,12 @@ __global__ void __launch_bounds__(128) k_events(const __grid_constant__ MoveArgs
     T* const uzp = static_cast<T*>(a.uz);
     const unsigned long long lane = threadIdx.x & 31;
     const unsigned long long per = min(32ull, (n + kEventSpread - 1) / kEventSpread);
-    const unsigned long long stride = (unsigned long long)gridDim.x * (blockDim.x >> 5) * per;
-    for (unsigned long long w = ((unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * per;
-         w < n; w += stride) {
+    const unsigned split = per < 32ull ? 2 : 0;  // log2 of the warps a group has
+    const unsigned wi = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    // (a grid is at least 32 blocks of four warps: the stride is a multiple of four warps)
+    const unsigned long long stride = (unsigned long long)(gridDim.x * (blockDim.x >> 5) >> split) * per;
+    const int role = split ? (int)(wi & 3u) : kRoleAll;
+    for (unsigned long long w = (unsigned long long)(wi >> split) * per; w < n; w += stride) {
         const unsigned long long i = w + lane;
         int ckey = -1, wkey = -1;  // collision counter, wall counter
         bool ok = lane < per && i < n;
@@ -302,7 +316,9 @@ __global__ void __launch_bounds__(128) k_events(const __grid_constant__ MoveArgs
             const int j0 = (int)((uint32_t)a.cell[slot] & kCellMask);
             if (kind == kRareCandidate && in_range(a.err, j0, 0, P.ncells)) {
                 const uint4 wd = draw(id, step, kRngCollide, P.key0, P.key1);
-                const int p = collide<T>(a, P, s, id, step, j0, f, vx, vy, vz, wd.y, wd.z, slot);
+                const int p = role == kRoleWall ? -1
+                                                : collide<T>(role, a, P, s, id, step, j0, f, vx, vy, vz,
+                                                             wd.y, wd.z, slot);
                 if (p >= 0) {
                     uxp[slot] = vx;
                     uyp[slot] = vy;
@@ -310,10 +326,12 @@ __global__ void __launch_bounds__(128) k_events(const __grid_constant__ MoveArgs
                     ckey = P.inst * kMaxProc + p;
                 }
                 // a candidate is followed by a test on the next own step: drawn now
-                const int ks = P.nstep;
-                const int64_t q = ks == 1 ? step + 1 : (step + 1) / ks;  // own step q - 1
-                a.cell[slot] = test_word(P, id, j0, q);
-            } else if (kind == kRareWallLow || kind == kRareWallHigh) {
+                if (role <= kRoleWall) {
+                    const int ks = P.nstep;
+                    const int64_t q = ks == 1 ? step + 1 : (step + 1) / ks;  // own step q - 1
+                    a.cell[slot] = test_word(P, id, j0, q);
+                }
+            } else if (role <= kRoleWall && (kind == kRareWallLow || kind == kRareWallHigh)) {
                 int j = kind == kRareWallLow ? -1 : P.ncells;
                 wkey = 2 * s + (kind == kRareWallLow ? 0 : 1);
                 if (wall_event<T>(a, P, s, id, step, j, f, vx, vy, vz) == 1) {

@@ -202,9 +202,7 @@ template <> struct Prec<double> {
     static __device__ __forceinline__ double uni(uint32_t w) { return ((double)w + 0.5) * 0x1p-32; }
     static __device__ __forceinline__ void sincos2pi(double u, double* s, double* c)
     {
-        const double th = 6.283185307179586476925286766559 * u;
-        *s = sin(th);
-        *c = cos(th);
+        sincospi(2.0 * u, s, c);  // (2 u is exact, so no rounding of 2 pi u precedes it)
     }
     static __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
     static __device__ __forceinline__ double log_(double x) { return log(x); }
