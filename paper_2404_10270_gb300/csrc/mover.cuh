@@ -75,6 +75,7 @@ struct MoveArgs {
     const int64_t* tile_start;          // nseg+1 prefix of tiles
     const int64_t* seg_nmove;           // slots of each segment moved this step
     int chunk;                          // consecutive tiles a warp of k_move takes at a time
+                                        // (k_move_sort: rounds of a block's tiles)
     unsigned long long* seg_n;          // slots in use (appends for created particles)
     unsigned long long* seg_live;       // live particles
     const void* accel;                  // T pairs (A_j, A_{j+1} - A_j), segment node arrays
@@ -1158,7 +1159,8 @@ k_move_sort(const __grid_constant__ MoveArgs a)
     SegFast F = {0, 0u, 0u, false};
     // every warp of the block walks the same chunks, so the barriers below match
     int parity = 0;
-    for (int64_t chunk = blockIdx.x; chunk * NW < total; chunk += gridDim.x, parity ^= 1) {
+    int64_t chunk = (int64_t)blockIdx.x * a.chunk;
+    for (int left = a.chunk; chunk * NW < total; parity ^= 1) {
         int* const wseg = wsum + parity * 3 * NW;
         int* const wmin = wseg + NW;
         int* const wmax = wmin + NW;
@@ -1420,6 +1422,11 @@ k_move_sort(const __grid_constant__ MoveArgs a)
             }
         }
         // 6. deposit of the new positions (that of a segment that rests stands)
+        ++chunk;
+        if (--left == 0) {  // on to the block's next rounds
+            left = a.chunk;
+            chunk += (int64_t)(gridDim.x - 1) * a.chunk;
+        }
         if (SUB && !moves) continue;
         int jd[4];
         Q qr[4];

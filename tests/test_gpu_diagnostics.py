@@ -1,5 +1,5 @@
 """pic_moments from one packet of a launch per call: the potential's two-level scan at the
-sizes around its chunks of 256 nodes, packets too large for the pinned copy, calls that
+sizes around its chunks of 256 nodes and the one-block field phase's 1,024, packets too large for the pinned copy, calls that
 skip arrays, and the kinetic energy over ragged particle counts."""
 import ctypes as C
 
@@ -14,7 +14,7 @@ pytestmark = [pytest.mark.gpu, requires_gpu]
 
 
 @pytest.mark.parametrize("smooth", [0, 1])
-@pytest.mark.parametrize("ncells", [1, 2, 255, 256, 257, 511, 40001])
+@pytest.mark.parametrize("ncells", [1, 2, 255, 256, 257, 511, 1022, 1023, 1024, 40001])
 def test_diagnostics_match_the_oracle(ncells, smooth):
     """Potential and densities of the load's deposit (the oracle's field phase is exact to its
     final rounding) and the kinetic energy summed in numpy's longdouble."""
