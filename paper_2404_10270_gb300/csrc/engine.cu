@@ -587,9 +587,13 @@ bool full_step(const pic_handle* h, int64_t n)
 // FP64 1.41 (16 tiles; 8: 1.43) against 1.47; 128 magnetized instances, FP32: 0.938 against
 // 1.060.  Below chunk_rounds tiles per resident warp the resident grid wins, whose warps
 // are set up once (98 M particles, 158 tiles a warp: 389 against 392 us a step; 49 M: 199
-// against 207; 30 M: 131 against 133), and so it does for the FP64 Boris form, which the
-// FP64 pipe bounds.
+// against 207; 30 M: 131 against 133).  The FP64 Boris form, which the FP64 pipe bounds,
+// wants its tiles spread evenly over the SMs: a block for every NT/32 tiles (from
+// kBorisRounds tiles per resident warp, twice as many) instead of the resident grid, whose
+// warps' tile counts differ by one (1.6 M particles, 3.5 tiles a warp: 78.1 us a step
+// against 80.6, 2 tiles 81.1; 39 M: 1,107 at one, 1,099 at two against 1,136).
 constexpr int kMoveChunk = 8;
+constexpr int64_t kBorisRounds = 16;
 // The sort step in the same manner: a block takes kSortChunk consecutive rounds of its
 // NT/32 tiles and ends.  196.6 M particles: FP32 2.30 -> 2.18 ms (8 rounds 2.21), FP64 4.01 ->
 // 3.83; 49 M FP32 559 -> 550 us (8: 568).  From kSortRounds tiles per resident warp.
@@ -635,13 +639,16 @@ int launch_move(pic_handle* h, bool move, int phase = kPlain)
         const int nt = sort ? h->nt_sort : h->nt;
         int grid = sort ? h->grid_sort : full ? h->grid_full : h->grid_move;
         const int64_t nw = nt / 32;
+        const bool boris64 = !sort && mag && h->precision == PIC_FP64;
         if (sort) {
             if (h->max_tiles >= std::min(h->chunk_rounds, kSortRounds) * nw * grid) a.chunk = kSortChunk;
-        } else if (h->max_tiles >= h->chunk_rounds * nw * grid && !(mag && h->precision == PIC_FP64)) {
+        } else if (boris64) {
+            a.chunk = h->max_tiles >= std::min(h->chunk_rounds, kBorisRounds) * nw * grid ? 2 : 1;
+        } else if (h->max_tiles >= h->chunk_rounds * nw * grid) {
             a.chunk = h->precision == PIC_FP64 ? 2 * kMoveChunk : kMoveChunk;
         }
         const int64_t blocks = (h->max_tiles + nw * a.chunk - 1) / (nw * a.chunk);
-        if (a.chunk > 1 || blocks < grid) grid = (int)std::max<int64_t>(blocks, 1);
+        if (a.chunk > 1 || boris64 || blocks < grid) grid = (int)std::max<int64_t>(blocks, 1);
         h->kernels += 1;
         const cudaError_t e =
             h->precision == PIC_FP64
