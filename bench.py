@@ -45,15 +45,16 @@ MOVER_BYTES = {"f32": 24, "f64": 40}
 # this GPU) x 152 SMs x 2.07 GHz.  The form is reported against whichever of the FP64
 # pipe and HBM it uses the larger fraction of.
 FP64_OPS_PER_PARTICLE = 3
-# With B != 0 (Boris): gather 1, half step 1, v + a/2 1, the two cross-product updates
-# 6 x 2 fused multiply-adds, the last half step 1, the move 1.
-FP64_OPS_PER_PARTICLE_BORIS = 17
+# With B != 0 (Boris) in the x-y plane, as in every workload here: gather 1 (of half the
+# acceleration), v + a/2 1, the two cross-product updates 4 x 2 fused multiply-adds, the last
+# half step 1, the move 1.
+FP64_OPS_PER_PARTICLE_BORIS = 12
 FP64_PEAK_INSTR_PER_S = 2 * 152 * 2.07e9
 # Mover threads per block of the 196.6 M-particle workload in both forms (the step that
-# ends a sort cycle has its own block size, 128): measured 0.856 against 0.873 ms per
-# step at 256 in FP32, 1.644 against 1.663 in FP64.  The subcycled variant and the
-# paper's test case keep 256 (their best).
-LARGE_BLOCK = 512
+# ends a sort cycle has its own block size, 128): with warps that take chunks of tiles, small
+# blocks follow the store most closely (0.748 / 0.764 / 0.770 ms per step at 128 / 256 / 512 in
+# FP32, 1.52 / 1.56 / 1.61 in FP64).  The subcycled variant and the paper's test case keep 256.
+LARGE_BLOCK = 128
 
 
 def peaks():
