@@ -809,7 +809,7 @@ void set_block(pic_handle* h, int nt)
     h->grid_full = grid(MoveMode::kFull);
     // tiles are fetched ahead where a resident warp has several of them
     h->grid_move = grid(MoveMode::kAhead);
-    h->mode = h->max_tiles >= h->ahead_tiles * h->grid_move * (nt / 32) ? MoveMode::kAhead : MoveMode::kDirect;
+    h->mode = !h->any_mag && h->max_tiles >= h->ahead_tiles * h->grid_move * (nt / 32) ? MoveMode::kAhead : MoveMode::kDirect;
     if (h->mode == MoveMode::kDirect) h->grid_move = grid(MoveMode::kDirect);
     // (the sort step's variant with the y coordinates of 2-D species holds more shared
     // memory a block; its block size is its own)

@@ -532,17 +532,17 @@ __device__ __forceinline__ void push(const SegParams& P, bool smag, T acc, T& ux
 // for them.  Once its instructions had gone from 448 to 289 a tile the FP32 mover waited
 // for HBM with 46 warps' loads in flight (0.730 ms for 196.6 M particles); with the ring
 // and kMoveChunk (engine.cu) it takes 0.64-0.65 ms, 6.1 TB/s of the 20 B a particle it
-// moves in fact.  One stage: the cell words, off, ux (and uy, uz) of a warp's tile.
-template <typename T, bool MAG>
+// moves in fact.  One stage: the cell words, off and ux of a warp's tile.
+template <typename T>
 struct TileRing {
-    static constexpr int words = 128 + (MAG ? 4 : 2) * 128 * (int)(sizeof(T) / 4);  // one stage
+    static constexpr int words = 128 + 2 * 128 * (int)(sizeof(T) / 4);  // one stage
     static constexpr size_t bytes(int nt) { return (size_t)(nt / 32) * 2 * words * 4; }
 };
 // Dynamic shared memory of a block of the mover: the rings of the variants that fetch ahead.
-template <typename T, bool MAG, MoveMode MODE>
+template <typename T, MoveMode MODE>
 constexpr size_t ring_bytes(int nt)
 {
-    return MODE == MoveMode::kAhead ? TileRing<T, MAG>::bytes(nt) : 0;
+    return MODE == MoveMode::kAhead ? TileRing<T>::bytes(nt) : 0;
 }
 // L2 policy of streamed reads: evict first (as the 128-bit loads' hint).
 __device__ __forceinline__ uint64_t stream_policy()
@@ -876,8 +876,10 @@ __device__ __forceinline__ void rare_quad(const MoveArgs& a, int s, bool smag, i
 // MIXED (with MAG): the batch mixes magnetized and unmagnetized instances, so the push is
 // chosen per segment.  MODE: kDirect loads a tile when its turn comes, for batches whose
 // warps have a tile or two (a ring of two 16 KB stages a block buys nothing there and its
-// set-up costs 1.5 us a step) and for the FP64 Boris form (4.6 KB a tile, bound by the FP64
-// pipe); kAhead fetches one tile ahead (TileRing); kFull is the variant of large batches
+// set-up costs 1.5 us a step) and for the Boris form (5 to 9 KB of ring a warp; 31 M
+// particles in 26 magnetized instances, FP32: 284 us a step direct, 310 fetched ahead, 125 M
+// the same either way; the FP64 one is bound by the FP64 pipe);
+// kAhead fetches one tile ahead (TileRing); kFull is the variant of large batches
 // for the steps on which the clocks of a whole species test (the multiples of kGapMax, the
 // first step after a load):
 // the quad's ids are read with its state and its four draws and table lookups go side by
@@ -894,6 +896,7 @@ k_move(const __grid_constant__ MoveArgs a)
     using Q = typename Prec<T>::Q;
     using T2 = typename Prec<T>::T2;
     constexpr bool PF = MODE == MoveMode::kAhead, FULL = MODE == MoveMode::kFull;
+    static_assert(!(PF && MAG), "the Boris form loads directly");
     const int lane = threadIdx.x & 31;
     T* const offp = static_cast<T*>(a.off);
     T* const uxp = static_cast<T*>(a.ux);
@@ -936,7 +939,7 @@ k_move(const __grid_constant__ MoveArgs a)
         ahead = ahead0 + (int64_t)tile * 128;
     };
     extern __shared__ __align__(16) uint32_t s_ring[];
-    constexpr int SW = TileRing<T, MAG>::words;
+    constexpr int SW = TileRing<T>::words;
     uint32_t* const ring = s_ring + (threadIdx.x >> 5) * 2 * SW;
     const uint32_t ring_at = PF ? (uint32_t)__cvta_generic_to_shared(ring) : 0u;
     const uint64_t policy = PF ? stream_policy() : 0ull;
@@ -946,10 +949,6 @@ k_move(const __grid_constant__ MoveArgs a)
             copy_quad(d, a.cell + ahead, policy);
             copy_quad(d + 512, offp + ahead, policy);
             copy_quad(d + 512 + 128 * sizeof(T), uxp + ahead, policy);
-            if (MAG) {
-                copy_quad(d + 512 + 256 * sizeof(T), uyp + ahead, policy);
-                copy_quad(d + 512 + 384 * sizeof(T), uzp + ahead, policy);
-            }
         }
         copy_commit();
     };
@@ -986,10 +985,6 @@ k_move(const __grid_constant__ MoveArgs a)
                 c[0] = cc.x; c[1] = cc.y; c[2] = cc.z; c[3] = cc.w;
                 take_quad(w + 128, f);
                 take_quad(w + 128 + 32 * sizeof(T), ux);
-                if (MAG) {
-                    take_quad(w + 128 + 64 * sizeof(T), uy);
-                    take_quad(w + 128 + 96 * sizeof(T), uz);
-                }
             }
         } else if (act) {
             const int4 cc = __ldcs(reinterpret_cast<const int4*>(a.cell + slot));

@@ -9,7 +9,7 @@ namespace {
 template <int NT, bool MAG, bool MOVE, bool SUB, bool MIXED, MoveMode MODE>
 cudaError_t launch(const MoveArgs& a, int grid, cudaStream_t st)
 {
-    k_move<float, NT, MAG, MOVE, SUB, MIXED, MODE><<<grid, NT, ring_bytes<float, MAG, MODE>(NT), st>>>(a);
+    k_move<float, NT, MAG, MOVE, SUB, MIXED, MODE><<<grid, NT, ring_bytes<float, MODE>(NT), st>>>(a);
     return cudaGetLastError();
 }
 
@@ -17,7 +17,8 @@ template <int NT, bool SUB, MoveMode MODE>
 cudaError_t go_sub(const MoveArgs& a, bool mag, bool mixed, int grid, cudaStream_t st)
 {
     if (!mag) return launch<NT, false, true, SUB, false, MODE>(a, grid, st);
-    constexpr MoveMode M = MODE;
+    // (the Boris form loads directly, see k_move)
+    constexpr MoveMode M = MODE == MoveMode::kAhead ? MoveMode::kDirect : MODE;
     return mixed ? launch<NT, true, true, SUB, true, M>(a, grid, st)
                  : launch<NT, true, true, SUB, false, M>(a, grid, st);
 }
@@ -46,7 +47,7 @@ template <int NT, bool MAG, bool SUB, bool MIXED, MoveMode MODE>
 int resident_one()
 {
     const auto k = k_move<float, NT, MAG, true, SUB, MIXED, MODE>;
-    const int sm = (int)ring_bytes<float, MAG, MODE>(NT);
+    const int sm = (int)ring_bytes<float, MODE>(NT);
     int n = 0;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, NT, sm);
@@ -56,7 +57,8 @@ template <int NT, bool SUB, MoveMode MODE>
 int resident(bool mag)
 {
     if (!mag) return resident_one<NT, false, SUB, false, MODE>();
-    constexpr MoveMode M = MODE;
+    // (the Boris form loads directly, see k_move)
+    constexpr MoveMode M = MODE == MoveMode::kAhead ? MoveMode::kDirect : MODE;
     if (resident_one<NT, true, SUB, true, M>() == 0) return 0;
     return resident_one<NT, true, SUB, false, M>();
 }

@@ -9,7 +9,7 @@ namespace {
 template <int NT, bool MAG, bool MOVE, bool SUB, bool MIXED, MoveMode MODE>
 cudaError_t launch(const MoveArgs& a, int grid, cudaStream_t st)
 {
-    k_move<double, NT, MAG, MOVE, SUB, MIXED, MODE><<<grid, NT, ring_bytes<double, MAG, MODE>(NT), st>>>(a);
+    k_move<double, NT, MAG, MOVE, SUB, MIXED, MODE><<<grid, NT, ring_bytes<double, MODE>(NT), st>>>(a);
     return cudaGetLastError();
 }
 
@@ -47,7 +47,7 @@ template <int NT, bool MAG, bool SUB, bool MIXED, MoveMode MODE>
 int resident_one()
 {
     const auto k = k_move<double, NT, MAG, true, SUB, MIXED, MODE>;
-    const int sm = (int)ring_bytes<double, MAG, MODE>(NT);
+    const int sm = (int)ring_bytes<double, MODE>(NT);
     int n = 0;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, NT, sm);
