@@ -154,11 +154,10 @@ struct pic_handle {
     bool hist_ready = false;
     int grid_sort = 0;
     int grid_full = 0;  // grid of the mover's kFull variant
-    // threads per block of the step that ends a sort cycle, apart from the other steps':
-    // its four block-wide barriers a chunk cost less in small blocks, while the plain
-    // mover gains from large ones (196.6 M particles, FP32: the sort step 2.22 / 2.31 /
-    // 2.57 ms at 128 / 256 / 512 threads, the plain mover 0.783 / 0.771 / 0.754 ms);
-    // `$BITPIC_SORT_BLOCK` (128, 256 or 512) overrides it
+    // threads per block of the step that ends a sort cycle, apart from the other steps': its
+    // four block-wide barriers a round cost less in small blocks (196.6 M particles: 2.18 /
+    // 2.27 ms at 128 / 256 threads in FP32, 3.83 / 4.14 in FP64); `$BITPIC_SORT_BLOCK` (128,
+    // 256 or 512) overrides it
     int nt_sort = 128;
     int state = PIC_OK;
     std::string last_error;
