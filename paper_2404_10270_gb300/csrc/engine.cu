@@ -565,9 +565,10 @@ FieldArgs field_args(pic_handle* h)
 
 // Whether the mover of step n takes its kFull variant: the clocks of a whole species may
 // test, after a load (any batch) or when the species' own step is a multiple of kGapMax
-// (large batches).  The other variants handle such a step too, one particle at a time:
-// below some 16 M slots that costs less than it saves to keep the step inside a captured
-// window (1.6 M particles: under 1 % of the time, averaged over 127 steps).
+// (large batches).  The other variants draw in place, after the tile, and below some 16 M
+// slots that keeps the step inside a captured window at the same price (14.4 M particles on
+// 65,536 cells, FP32: 144 us on such a step, 121 in kFull, 58 on the others; averaged over
+// 127 steps 76.2 against 76.6 us a step, 1.0 M on 256 cells 19.0 against 19.2).
 bool full_step(const pic_handle* h, int64_t n)
 {
     for (int K : h->collide_nsteps)

@@ -21,7 +21,7 @@
 // 128-bit accesses.  The particle id is not streamed: it is read only at clock test
 // steps (once per 127 steps per particle) and by the event kernel.  Warps walk the
 // tiles of all segments independently, with no block-level barrier, so an SM keeps
-// the loads of many tiles in flight.  The loop has no calls: the rare events
+// the loads of many tiles in flight.  The common path has no calls: the rare events
 // (collision candidates, wall hits) go to a queue that the event kernel
 // (events.cuh) works through after the mover, so the common path keeps its whole
 // state in registers.  Velocity changes do not move a particle, so a candidate is
@@ -587,6 +587,16 @@ __device__ __forceinline__ void queue_rare(const MoveArgs& a, int s, int64_t slo
     else set_error(a.err, kErrEvents);
 }
 
+// The clock bits that follow a test at own step mown whose draw gives `run` candidate-free
+// own steps; dgrid: the own steps to the species' next multiple of kGapMax.  now: a
+// candidate on this very step.
+__device__ __forceinline__ uint32_t clock_after_test(int run, int64_t mown, int dgrid, bool& now)
+{
+    const int g = min(run, dgrid);
+    now = g == 0;
+    return clock_bits(now ? mown + 1 : mown + g, g > 0 && g < dgrid);
+}
+
 // Steps 1-5 of the time step for one live particle: gather, push, move, walls,
 // collision clock.  c, f, u* hold its state on entry and its new state on exit (cell
 // word -1: left through a wall).  mown is the species' own index of this step (its
@@ -643,10 +653,9 @@ __device__ __forceinline__ int particle_step(const MoveArgs& a, const SegParams&
             // candidate and puts its outcome in the clock)
             clk = (uint32_t)((mown + 1) & (int64_t)kClockDue);
         } else {
-            const int g = min(run(), dgrid);
-            if (g == 0) ev = (int)kRareCandidate;
-            const int64_t due = g == 0 ? mown + 1 : mown + g;
-            clk = (uint32_t)(due & (int64_t)kClockDue) | (g > 0 && g < dgrid ? kClockPending : 0u);
+            bool now;
+            clk = clock_after_test(run(), mown, dgrid, now) >> kClockShift;
+            if (now) ev = (int)kRareCandidate;
         }
     }
     c = (int)((uint32_t)j | (clk << kClockShift));
@@ -722,8 +731,9 @@ struct SegFast {
 // instructions as much as by HBM, so this runs without branches: the cell is the word's
 // low bits, so the new word is the old one plus the cells crossed.  due: a clock of the
 // quad is due (quad_due).  Returns true when a particle of the quad is not of that kind
-// (a wall, an offset that rounded up to 1, a velocity that is not finite): the whole quad is then done over by rare_quad from the state in memory, which must not
-// have been written before.
+// (a wall, an offset that rounded up to 1, a velocity that is not finite): the whole quad is
+// then done over by rare_quad from the state in memory, which must not have been written
+// before.
 template <typename T, bool MAG>
 __device__ __forceinline__ bool quad_fast(const SegParams& P, const SegFast& F, bool smag,
                                           const typename Prec<T>::T2* __restrict__ accn, int c[4],
@@ -783,25 +793,25 @@ __device__ __forceinline__ bool quad_fast(const SegParams& P, const SegFast& F, 
     return rare;
 }
 
-// A quad of the common path with a due clock: one bit per pending collision candidate,
+// A quad of the common path with a due clock: in bits 0-3 its pending collision candidates,
 // whose clocks are set to the test that follows (the event kernel draws it when it takes
-// the candidate); -1 when a clock tests, which is left to rare_quad.
+// the candidate), in bits 4-7 the clocks that test on this step, left to test_clock.
 __device__ __forceinline__ int quad_due(const SegFast& F, int c[4])
 {
     constexpr uint32_t pend = kClockPending << kClockShift;
     const uint32_t mask = F.clkmask | pend, next = (F.due + (1u << kClockShift)) & F.clkmask;
-    bool test = false;
+    int ev = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) test |= c[k] >= 0 && (((uint32_t)c[k] ^ F.due) & mask) == 0u;
-    if (test) return -1;
-    int cand = 0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-        if (c[k] >= 0 && (((uint32_t)c[k] ^ F.due) & mask) == pend) {
-            cand |= 1 << k;
+    for (int k = 0; k < 4; ++k) {
+        if (c[k] < 0) continue;
+        const uint32_t d = ((uint32_t)c[k] ^ F.due) & mask;
+        if (d == 0u) ev |= 16 << k;
+        if (d == pend) {
+            ev |= 1 << k;
             c[k] = (int)(((uint32_t)c[k] & kCellMask) | next);
         }
-    return cand;
+    }
+    return ev;
 }
 
 // The species' own index of step `step` (its clock's time) and the own steps to its next
@@ -810,6 +820,66 @@ __device__ __forceinline__ void own_time(const SegParams& P, int64_t step, int64
 {
     mown = P.nstep == 1 ? step : (step + 1) / P.nstep - 1;
     dgrid = kGapMax - (int)(mown % kGapMax);
+}
+
+// The clock test of one particle of the common path, whose word after the move is c: the
+// word with the clock that follows, its candidate of this step queued at slot `to` (-1:
+// none, nothing is queued).
+__device__ __forceinline__ int test_clock(const MoveArgs& a, const SegParams& P, int s, int64_t step,
+                                          int64_t mown, int dgrid, uint32_t id, int c, int64_t to)
+{
+    bool now;
+    const uint32_t clk = clock_after_test(
+        gap_steps(P.gap, P.glog, draw(id, step, kRngCollide, P.key0, P.key1).x), mown, dgrid, now);
+    if (now && to >= 0) queue_rare(a, s, to, kRareCandidate);
+    return (int)(((uint32_t)c & kCellMask) | clk);
+}
+
+// The tests are called, not inlined: inlined, their registers moved the schedule of the
+// loop (196.6 M particles, FP32: mover 650 against 646 us, the sort step 2.28 against
+// 2.22 ms); and with them called the Boris form wants rare_quad called too (39 M particles
+// in FP32: 230 us, inlined 250), the others not (650 against 647).
+//
+// The clock tests of a quad that is in memory again after its step (plain step), `test` a bit
+// per quad position.  Only the clocks are left to do: the quad's move and its share of the
+// warp's deposit are the common path's.  (Doing such quads over one particle at a time, with
+// two 64-bit atomics each, took 5.5 ms for the 14.3 M particles of a 256-cell plasma on the
+// steps on which every clock tests, and 72 us on the others.)
+static __device__ __noinline__ void test_quad(const MoveArgs& a, int s, int64_t step, int64_t slot,
+                                              int test)
+{
+    const SegParams& P = a.seg[s];
+    int64_t mown;
+    int dgrid;
+    own_time(P, step, mown, dgrid);
+    const uint4 id = __ldcs(reinterpret_cast<const uint4*>(a.id + slot));
+    const int4 c = *reinterpret_cast<const int4*>(a.cell + slot);
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k)
+        if (test >> k & 1)
+            a.cell[slot + k] = test_clock(a, P, s, step, mown, dgrid,
+                                          k == 0 ? id.x : k == 1 ? id.y : k == 2 ? id.z : id.w,
+                                          k == 0 ? c.x : k == 1 ? c.y : k == 2 ? c.z : c.w, slot + k);
+}
+
+// The same of a quad staged for the sort at the places pk of the chunk's arrays (-1: none);
+// `ev` as quad_due gives it.
+static __device__ __noinline__ void test_staged(const MoveArgs& a, int s, int64_t step, int ev, short4 pk,
+                                                int* s_cell, const uint32_t* s_id,
+                                                const uint32_t* s_dst)
+{
+    const SegParams& P = a.seg[s];
+    int64_t mown;
+    int dgrid;
+    own_time(P, step, mown, dgrid);
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+        const int p = k == 0 ? pk.x : k == 1 ? pk.y : k == 2 ? pk.z : pk.w;
+        if (!(ev >> k & 16) || p < 0) continue;
+        const uint32_t d = s_dst[p];
+        s_cell[p] = test_clock(a, P, s, step, mown, dgrid, s_id[p], s_cell[p],
+                               d == 0xFFFFFFFFu ? (int64_t)-1 : P.base + (int64_t)d);
+    }
 }
 
 // One particle of a quad the common path left, from the state in memory at slot g:
@@ -866,12 +936,20 @@ __device__ __forceinline__ void rare_quad(const MoveArgs& a, int s, bool smag, i
     }
 }
 
+// rare_quad called: the Boris form's loop, whose registers are scarce (see test_quad).
+template <typename T>
+static __device__ __noinline__ void rare_quad_boris(const MoveArgs& a, int s, bool smag, int64_t step,
+                                                    int64_t slot)
+{
+    rare_quad<T, true>(a, s, smag, step, slot);
+}
+
 // The fused time step.  Work unit: a warp tile of 32 quads (128 consecutive particles
 // of one segment); each lane owns one quad and moves it with 128-bit accesses.  Warps
 // walk the tiles of all segments independently (no block-level barrier), so every SM
 // keeps many tiles' loads in flight.  The gather reads each particle's node pair with
-// one vector load (the node arrays are small and stay in L1/L2).  The loop is free of
-// calls; walls and collision candidates are queued for the event kernel.
+// one vector load (the node arrays are small and stay in L1/L2).  The common
+// path is free of calls; walls and collision candidates are queued for the event kernel.
 // SUB: some species of the batch is subcycled (else every segment moves every step).
 // MIXED (with MAG): the batch mixes magnetized and unmagnetized instances, so the push is
 // chosen per segment.  MODE: kDirect loads a tile when its turn comes, for batches whose
@@ -883,8 +961,8 @@ __device__ __forceinline__ void rare_quad(const MoveArgs& a, int s, bool smag, i
 // for the steps on which the clocks of a whole species test (the multiples of kGapMax, the
 // first step after a load):
 // the quad's ids are read with its state and its four draws and table lookups go side by
-// side before the physics; the other steps' variant leaves such quads, one particle at a
-// time, to rare_quad, which gives the same results.  A segment that rests on this step
+// side before the physics; the other steps' variant draws them one after another once the
+// tile is done (test_quad), with the same results.  A segment that rests on this step
 // (subcycling, a neutral particle target) keeps its deposit, so its tiles are skipped, or
 // only counted per cell on the step before a sort: the 30,011-cell plasma with ions moved
 // every fourth step (42 M particles, FP32) went from 212 to 183 us a step.  (The step
@@ -1012,7 +1090,9 @@ k_move(const __grid_constant__ MoveArgs a)
             own_time(P, step, mown, dgrid);
             F.set(P, mown);
         }
-        bool rare = false;
+        // what the quad leaves until the tile is done: -1 all of it (rare_quad), else a bit per
+        // clock that tests (test_quad)
+        int todo = 0;
         if (MOVE && (!SUB || moves)) {
             const SegParams& P = a.seg[s];
             bool moved = false;
@@ -1042,15 +1122,16 @@ k_move(const __grid_constant__ MoveArgs a)
                 }
             } else {
                 bool due;
-                rare = quad_fast<T, MAG>(P, F, smag, static_cast<const T2*>(a.accel) + node0, c, f,
-                                         ux, uy, uz, moved, due, scr) && act;
+                const bool rare = quad_fast<T, MAG>(P, F, smag, static_cast<const T2*>(a.accel) + node0,
+                                                    c, f, ux, uy, uz, moved, due, scr);
+                if (rare && act) todo = -1;
                 if (due && act && !rare) {
-                    const int cand = quad_due(F, c);
-                    rare = cand < 0;
+                    const int ev = quad_due(F, c);
+                    todo = ev >> 4;
                     moved = true;
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        if (!rare && (cand >> k & 1)) queue_rare(a, s, slot + k, kRareCandidate);
+                        if (ev >> k & 1) queue_rare(a, s, slot + k, kRareCandidate);
                 }
             }
             // the cell words go back only where one of them changed (a cell crossing, a
@@ -1058,7 +1139,7 @@ k_move(const __grid_constant__ MoveArgs a)
             // per 32-byte sector (two lanes) so that memory sees whole sectors
             const int chg = moved ? 1 : 0;
             const bool wcell = (chg | __shfl_xor_sync(0xffffffffu, chg, 1)) != 0;
-            if (act && !rare) {
+            if (act && todo >= 0) {
                 if (wcell)
                     __stcs(reinterpret_cast<int4*>(a.cell + slot), make_int4(c[0], c[1], c[2], c[3]));
                 st4(offp + slot, f);
@@ -1075,14 +1156,18 @@ k_move(const __grid_constant__ MoveArgs a)
         Q qr[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            jd[k] = rare ? -1 : (int)((uint32_t)c[k] & (kCellMask | 0x80000000u));
+            jd[k] = todo < 0 ? -1 : (int)((uint32_t)c[k] & (kCellMask | 0x80000000u));
             if (kChecked && jd[k] >= 0 && !in_range(a.err, jd[k], 0, a.seg[s].ncells)) jd[k] = -1;
             qr[k] = (Q)Prec<T>::qright(f[k]);
         }
         warp_deposit<Q, MOVE && SUB>(jd, qr, Prec<T>::S,
                                      MOVE && SUB && !moves ? nullptr : a.dep + node0,
                                      a.hist_out ? a.hist_out + node0 : nullptr, dwin);
-        if (!FULL && rare) rare_quad<T, MAG>(a, s, smag, step, slot);
+        if (!FULL && todo != 0) {
+            if (todo > 0) test_quad(a, s, step, slot, todo);
+            else if (MAG) rare_quad_boris<T>(a, s, smag, step, slot);
+            else rare_quad<T, MAG>(a, s, smag, step, slot);
+        }
     }
 }
 
@@ -1239,8 +1324,8 @@ k_move_sort(const __grid_constant__ MoveArgs a)
             bmax = __reduce_max_sync(FULL, mx);
         }
         const bool staged = one && bseg >= 0 && bmax - bmin < kSortSpan;
-        bool rare = false, moved = false;
-        int cand = 0;  // collision candidates of a quad that is not rare
+        bool moved = false;
+        int ev = 0;  // -1: a quad the common path left, else see quad_due
         const T2* const accn = static_cast<const T2*>(a.accel) + P.node;
         if (staged) {
             const SegParams& B = a.seg[bseg];
@@ -1287,11 +1372,9 @@ k_move_sort(const __grid_constant__ MoveArgs a)
             }
             if (!SUB || moves) {
                 bool due;
-                rare = quad_fast<T, MAG>(P, F, smag, accn, c, f, ux, uy, uz, moved, due, scr) && act;
-                if (due && act && !rare) {
-                    cand = quad_due(F, c);
-                    rare = cand < 0;
-                }
+                const bool rare = quad_fast<T, MAG>(P, F, smag, accn, c, f, ux, uy, uz, moved, due, scr);
+                if (rare && act) ev = -1;
+                if (due && act && !rare) ev = quad_due(F, c);
             }
             if (threadIdx.x < kSortSpan) gb[threadIdx.x] = gres;
             __syncthreads();
@@ -1314,10 +1397,13 @@ k_move_sort(const __grid_constant__ MoveArgs a)
                 if (YP) s_yp[p] = static_cast<const T*>(a.yp)[slot + k];
                 const int64_t r = (int64_t)gb[key[k]] + rank[k];
                 s_dst[p] = r < B.cap ? (uint32_t)r : 0xFFFFFFFFu;
-                if (!rare && (cand >> k & 1) && r < B.cap)
-                    queue_rare(a, bseg, B.base + r, kRareCandidate);
+                if (ev > 0 && (ev >> k & 1) && r < B.cap) queue_rare(a, bseg, B.base + r, kRareCandidate);
             }
-            if (rare) {
+            if (ev > 15)
+                test_staged(a, bseg, step, ev,
+                            make_short4((short)pk[0], (short)pk[1], (short)pk[2], (short)pk[3]), s_cell,
+                            s_id, s_dst);
+            if (ev < 0) {
                 int64_t mown;
                 int dgrid;
                 own_time(B, step, mown, dgrid);
@@ -1378,11 +1464,9 @@ k_move_sort(const __grid_constant__ MoveArgs a)
             }
             if (!SUB || moves) {
                 bool due;
-                rare = quad_fast<T, MAG>(P, F, smag, accn, c, f, ux, uy, uz, moved, due, scr) && act;
-                if (due && act && !rare) {
-                    cand = quad_due(F, c);
-                    rare = cand < 0;
-                }
+                const bool rare = quad_fast<T, MAG>(P, F, smag, accn, c, f, ux, uy, uz, moved, due, scr);
+                if (rare && act) ev = -1;
+                if (due && act && !rare) ev = quad_due(F, c);
             }
             int64_t to[4];
             sort_destinations(a, P, grp, rbase, had, to);
@@ -1393,12 +1477,22 @@ k_move_sort(const __grid_constant__ MoveArgs a)
                     if (to[k] >= 0)
                         static_cast<T*>(a.dyp)[to[k]] = static_cast<const T*>(a.yp)[slot + k];
             }
-            if (!rare && cand != 0) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if ((cand >> k & 1) && to[k] >= 0) queue_rare(a, s, to[k], kRareCandidate);
+            if (ev > 0) {
+                int64_t mown;
+                int dgrid;
+                own_time(P, step, mown, dgrid);
+#pragma unroll 1
+                for (int k = 0; k < 4; ++k) {
+                    const int64_t g = k == 0 ? to[0] : k == 1 ? to[1] : k == 2 ? to[2] : to[3];
+                    if (g < 0) continue;
+                    if (ev >> k & 1) queue_rare(a, s, g, kRareCandidate);
+                    if (ev >> k & 16)
+                        a.dcell[g] = test_clock(a, P, s, step, mown, dgrid,
+                                                k == 0 ? idq[0] : k == 1 ? idq[1] : k == 2 ? idq[2] : idq[3],
+                                                k == 0 ? c[0] : k == 1 ? c[1] : k == 2 ? c[2] : c[3], g);
+                }
             }
-            if (rare) {
+            if (ev < 0) {
                 // put right what the common path left, in the slots just written
                 int64_t mown;
                 int dgrid;
@@ -1433,7 +1527,7 @@ k_move_sort(const __grid_constant__ MoveArgs a)
         Q qr[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            jd[k] = rare ? -1 : (int)((uint32_t)c[k] & (kCellMask | 0x80000000u));
+            jd[k] = ev < 0 ? -1 : (int)((uint32_t)c[k] & (kCellMask | 0x80000000u));
             if (kChecked && jd[k] >= 0 && !in_range(a.err, jd[k], 0, P.ncells)) jd[k] = -1;
             qr[k] = (Q)Prec<T>::qright(f[k]);
         }
