@@ -325,7 +325,7 @@ __device__ __forceinline__ void st4(double* p, const double v[4])
 
 // Warp-level deposit of four particles per lane.  With Q = rint(f S) the charge of one
 // particle is S - Q on node j and Q on node j+1; a tile of 128 particles puts at most
-// 128 S on a node, so a node's sum fits 32 bits (FP64: two halves of 24 bits and up).  The
+// 128 S on a node, so a node's sum fits 32 bits (FP64: two words).  The
 // warp forms the sums of the nodes of its range [wmin, wmax + 1]; lane l then owns node
 // wmin + l and adds its sum to HBM with one 64-bit reduction (no return value, so nothing
 // waits on it).  A warp whose particles sit in a few cells (the store was sorted
@@ -335,21 +335,21 @@ __device__ __forceinline__ void st4(double* p, const double v[4])
 // adds each particle's two shares into a window of 32 nodes in shared memory (`win`, the
 // warp's own, zero outside this call; kDepReps copies side by side, a lane's by its
 // number, so that lanes in one cell seldom meet), which costs the same few instructions
-// whatever the spread; beyond 32 nodes every particle goes to HBM on its own.
+// whatever the spread; FP64 adds its count and its Q to its cell instead, two words where two
+// shares are four, and node i gets n_i S - R_i + R_{i-1} (n particles in the cell, R the sum
+// of their Q).  Beyond 32 nodes every particle goes to HBM on its own.
 // A negative jd marks an empty slot: as unsigned it is never the minimum of a live cell,
 // as signed never the maximum, and it matches no cell.
 // gdep null (OPT variants): only the counts, for a species whose deposit stands.
-// Register reductions up to this many cells (FP64: one more, its window costs four shared
-// atomics a particle).  196.6 M particles, FP32, 256-thread blocks: 0.644 ms at 2, 0.655 at
-// 3, 0.662 at 5; FP64, 512-thread blocks: 1.475 at 2, 1.435 at 3, 1.444 at 5.
-template <typename Q>
-struct DepLoop {
-    static constexpr int cells = sizeof(Q) == 4 ? 2 : 3;
-};
+// Register reductions up to kDepLoop cells: 196.6 M particles, FP32, 256-thread blocks: 0.644
+// ms at 2, 0.655 at 3, 0.662 at 5; FP64 1.384 at 2, 1.402 at 3, 1.409 at 4 (with a window of
+// four atomics a particle, two halves of two shares, 1.402 at its best, 3).
+constexpr int kDepLoop = 2;
 constexpr int kDepReps = 4;
 
-// Words of a warp's deposit window: 32 nodes of kDepReps copies (FP64: low halves, then
-// high halves; a half summed over a tile of 128 stays below 2^32).
+// Words of a warp's deposit window: 32 nodes of kDepReps copies.  FP64: 32 cells, first the
+// low 21 bits of Q above a count, then its high 27 bits; a copy sees at most 32 particles of
+// a tile, so the counts fit six bits, and either word's sum 32.
 template <typename Q>
 struct DepWin {
     static constexpr int words = 32 * kDepReps * (sizeof(Q) / 4);
@@ -365,13 +365,13 @@ __device__ __forceinline__ void dep_win_clear(uint32_t* win)
     __syncwarp();
 }
 
-// Sum of a lane's node copies in the window, which are cleared.
-__device__ __forceinline__ uint32_t dep_win_take(uint32_t* win)
+// A lane's copies in the window, which are cleared.
+__device__ __forceinline__ uint4 dep_win_take(uint32_t* win)
 {
     uint4* const p = reinterpret_cast<uint4*>(win) + (threadIdx.x & 31);
     const uint4 v = *p;
     *p = make_uint4(0u, 0u, 0u, 0u);
-    return (v.x + v.y) + (v.z + v.w);
+    return v;
 }
 
 template <typename Q, bool OPT = false>
@@ -381,7 +381,7 @@ __device__ __forceinline__ void warp_deposit(const int jd[4], const Q qr[4],
                                              unsigned* __restrict__ ghist,
                                              uint32_t* __restrict__ win)
 {
-    static_assert(kDepReps == 4, "dep_win_take reads a node's copies as one uint4");
+    static_assert(kDepReps == 4, "dep_win_take reads the copies as one uint4");
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned lmin = min(min((unsigned)jd[0], (unsigned)jd[1]), min((unsigned)jd[2], (unsigned)jd[3]));
@@ -393,7 +393,7 @@ __device__ __forceinline__ void warp_deposit(const int jd[4], const Q qr[4],
     if (ncell < 32) {
         if (!OPT || gdep) {
             unsigned long long tot = 0;  // the sum of node wmin + lane
-            if (ncell <= DepLoop<Q>::cells) {
+            if (ncell <= kDepLoop) {
                 Q left[4], carry = 0;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) left[k] = (Q)S - qr[k];
@@ -421,21 +421,31 @@ __device__ __forceinline__ void warp_deposit(const int jd[4], const Q qr[4],
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     if (jd[k] < 0) continue;
-                    uint32_t* const p = w + kDepReps * (jd[k] - wmin);
-                    const Q l = (Q)S - qr[k];
                     if (sizeof(Q) == 4) {
-                        atomicAdd(p, (uint32_t)l);
+                        uint32_t* const p = w + kDepReps * (jd[k] - wmin);
+                        atomicAdd(p, (uint32_t)S - (uint32_t)qr[k]);
                         atomicAdd(p + kDepReps, (uint32_t)qr[k]);
                     } else {
-                        atomicAdd(p, (uint32_t)((uint64_t)l & 0xFFFFFFu));
-                        atomicAdd(p + kDepReps, (uint32_t)((uint64_t)qr[k] & 0xFFFFFFu));
-                        atomicAdd(p + 32 * kDepReps, (uint32_t)((uint64_t)l >> 24));
-                        atomicAdd(p + 33 * kDepReps, (uint32_t)((uint64_t)qr[k] >> 24));
+                        // (Q = S, an offset that rounds up to 1: the next cell's, with Q = 0)
+                        const uint64_t q = (uint64_t)qr[k];
+                        uint32_t* const p = w + kDepReps * (jd[k] - wmin + (int)(q >> 48));
+                        atomicAdd(p, ((uint32_t)q & 0x1FFFFFu) << 6 | 1u);
+                        atomicAdd(p + 32 * kDepReps, (uint32_t)(q >> 21) & 0x7FFFFFFu);
                     }
                 }
                 __syncwarp();
-                tot = dep_win_take(win);
-                if (sizeof(Q) == 8) tot += (unsigned long long)dep_win_take(win + 32 * kDepReps) << 24;
+                if (sizeof(Q) == 4) {
+                    const uint4 v = dep_win_take(win);
+                    tot = (v.x + v.y) + (v.z + v.w);
+                } else {
+                    const uint4 a = dep_win_take(win), b = dep_win_take(win + 32 * kDepReps);
+                    const uint32_t n = (a.x & 63u) + (a.y & 63u) + (a.z & 63u) + (a.w & 63u);
+                    const uint32_t lo = (a.x >> 6) + (a.y >> 6) + (a.z >> 6) + (a.w >> 6);
+                    const uint64_t hi = ((uint64_t)b.x + b.y) + ((uint64_t)b.z + b.w);
+                    const unsigned long long R = (hi << 21) + lo;
+                    const unsigned long long prev = __shfl_up_sync(FULL, R, 1);
+                    tot = S * n - R + (lane > 0 ? prev : 0ull);
+                }
                 __syncwarp();
             }
             // (lanes past the range hold zeros)
