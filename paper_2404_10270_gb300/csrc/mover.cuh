@@ -1255,10 +1255,21 @@ struct SortSmem {
                                     (size_t)3 * kSortSpan * 4 + (size_t)2 * 3 * NW * 4;
 };
 
+// Resident blocks per SM the sort step is compiled for: registers before warps, since its
+// particles keep their velocities, ids and ranks beside the move (FP64 spilled 156 bytes at
+// 24 warps and 80 registers: 196.6 M particles 3.79 ms, 3.57 at 20 warps, 3.86 at 16; FP32 at
+// 32 warps and 64 registers 2.22, 2.20 at 28, 2.17 at 24; 39 M magnetized 577, 565, 549 us).
+// Larger blocks, which nothing but $BITPIC_SORT_BLOCK takes, keep the Boris form's warps.
+template <typename T, int NT>
+struct SortOccupancy {
+    static constexpr int warps = NT != 128 ? MoveOccupancy<T, true, NT>::warps : sizeof(T) == 8 ? 20 : 24;
+    static constexpr int blocks = warps / (NT / 32) > 0 ? warps / (NT / 32) : 1;
+};
+
 // YP: some species drifts in y (MoveArgs.yp): the y coordinates are sorted with the
 // particles (a separate variant: carrying them costs the others registers).
 template <typename T, int NT, bool MAG, bool SUB, bool MIXED, bool YP>
-__global__ void __launch_bounds__(NT, MoveOccupancy<T, true, NT>::blocks)
+__global__ void __launch_bounds__(NT, SortOccupancy<T, NT>::blocks)
 k_move_sort(const __grid_constant__ MoveArgs a)
 {
     using Q = typename Prec<T>::Q;
