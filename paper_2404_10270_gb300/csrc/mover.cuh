@@ -783,19 +783,45 @@ struct SegFast {
     }
 };
 
+// The particles of a quad that the common path moved through an absorbing or source wall:
+// their slots emptied and `walls` set, bit k at the low wall and bit 4+k at the high one.
+// Cell words as quad_fast leaves them (the cells crossed added, so that the low bits are the
+// cell's, of either sign).  False, with nothing changed, when the quad needs more than that:
+// an offset that rounded up to 1, a velocity that is not finite or takes a particle further
+// than the bits show.
+template <typename T>
+__device__ __forceinline__ bool quad_walls(int N, int c[4], const T f[4], const T ux[4], int& walls)
+{
+    constexpr int far = 1 << 20;  // (far_cells counts to twice that)
+    bool ok = N <= 2 * far;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) ok = ok && f[k] < T(1) && ux[k] < T(far) && ux[k] > T(-far);
+    if (!ok) return false;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int j = (int)((uint32_t)c[k] << (32 - kClockShift)) >> (32 - kClockShift);
+        if ((uint32_t)j < (uint32_t)N) continue;
+        c[k] = -1;
+        walls |= (j < 0 ? 1 : 16) << k;
+    }
+    return true;
+}
+
 // Steps 1-5 for the four particles of one quad (a lane's share of a tile), the common
 // case: live particles that stay inside the walls.  The mover is bound by its
 // instructions as much as by HBM, so this runs without branches: the cell is the word's
 // low bits, so the new word is the old one plus the cells crossed.  due: a clock of the
-// quad is due (quad_due).  Returns true when a particle of the quad is not of that kind
-// (a wall, an offset that rounded up to 1, a velocity that is not finite): the whole quad is
-// then done over by rare_quad from the state in memory, which must not have been written
-// before.
-template <typename T, bool MAG>
+// quad is due (quad_due), or a particle left through a wall (WALLS, quad_walls).  Returns true
+// when some particle needs more than that: the whole quad is then done over by rare_quad from
+// the state in memory, which must not have been written before.  (A wrapped particle is left
+// to it as well: with the others of its tile it would spread the warp's deposit from the
+// first cell to the last.)  WALLS: the plain push alone; in the Boris form and the sort step
+// the code costs the common path more registers than the rare quads cost.
+template <typename T, bool MAG, bool WALLS = false>
 __device__ __forceinline__ bool quad_fast(const SegParams& P, const SegFast& F, bool smag,
                                           const typename Prec<T>::T2* __restrict__ accn, int c[4],
                                           T f[4], T ux[4], T uy[4], T uz[4], bool& moved, bool& due,
-                                          double* scr)
+                                          int& walls, double* scr)
 {
     using T2 = typename Prec<T>::T2;
     // an empty slot is given a particle at rest in the first cell, its clock not due, and
@@ -841,6 +867,10 @@ __device__ __forceinline__ bool quad_fast(const SegParams& P, const SegFast& F, 
         if (sizeof(T) == 8 && dj != 0) cross |= 1u << k;
     }
     rare |= add_crossed(c, F.N, f, cross, scr);
+    if (WALLS && rare && P.bc != PIC_BC_PERIODIC) {
+        rare = !quad_walls<T>(F.N, c, f, ux, walls);
+        due |= walls != 0;
+    }
     if (empty) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
@@ -1179,16 +1209,20 @@ k_move(const __grid_constant__ MoveArgs a)
                 }
             } else {
                 bool due;
-                const bool rare = quad_fast<T, MAG>(P, F, smag, static_cast<const T2*>(a.accel) + node0,
-                                                    c, f, ux, uy, uz, moved, due, scr);
+                int walls = 0;
+                const bool rare = quad_fast<T, MAG, !MAG>(P, F, smag, static_cast<const T2*>(a.accel) + node0,
+                                                          c, f, ux, uy, uz, moved, due, walls, scr);
                 if (rare && act) todo = -1;
                 if (due && act && !rare) {
                     const int ev = quad_due(F, c);
                     todo = ev >> 4;
                     moved = true;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
+                    for (int k = 0; k < 4; ++k) {
                         if (ev >> k & 1) queue_rare(a, s, slot + k, kRareCandidate);
+                        if (!MAG && (walls >> k & 17))
+                            queue_rare(a, s, slot + k, walls >> k & 1 ? kRareWallLow : kRareWallHigh);
+                    }
                 }
             }
             // the cell words go back only where one of them changed (a cell crossing, a
@@ -1440,7 +1474,8 @@ k_move_sort(const __grid_constant__ MoveArgs a)
             }
             if (!SUB || moves) {
                 bool due;
-                const bool rare = quad_fast<T, MAG>(P, F, smag, accn, c, f, ux, uy, uz, moved, due, scr);
+                int walls = 0;
+                const bool rare = quad_fast<T, MAG>(P, F, smag, accn, c, f, ux, uy, uz, moved, due, walls, scr);
                 if (rare && act) ev = -1;
                 if (due && act && !rare) ev = quad_due(F, c);
             }
@@ -1532,7 +1567,8 @@ k_move_sort(const __grid_constant__ MoveArgs a)
             }
             if (!SUB || moves) {
                 bool due;
-                const bool rare = quad_fast<T, MAG>(P, F, smag, accn, c, f, ux, uy, uz, moved, due, scr);
+                int walls = 0;
+                const bool rare = quad_fast<T, MAG>(P, F, smag, accn, c, f, ux, uy, uz, moved, due, walls, scr);
                 if (rare && act) ev = -1;
                 if (due && act && !rare) ev = quad_due(F, c);
             }
