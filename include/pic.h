@@ -152,8 +152,9 @@ typedef struct {
                                    every collision clock tests; from $BITPIC_AHEAD_TILES
                                    (2) tiles of 128 particles per resident warp the mover
                                    fetches them ahead, and from $BITPIC_CHUNK_ROUNDS (200)
-                                   its warps take several consecutive tiles; this too
-                                   changes no result. */
+                                   its warps take several consecutive tiles;
+                                   $BITPIC_MOVE_BLOCKS bounds the mover's grid (tests; 0:
+                                   no bound); these too change no result. */
     const pic_instance* inst;   /* n_instances entries, copied */
     void* cuda_stream;          /* borrowed cudaStream_t; NULL = library-owned stream */
 } pic_config;

@@ -128,6 +128,7 @@ struct pic_handle {
     int64_t full_min = (int64_t)1 << 24;  // particle slots from which test steps take the kFull mover
     int64_t ahead_tiles = 2;    // tiles per resident warp from which the mover fetches them ahead
     int64_t chunk_rounds = 200; // tiles per resident warp from which its warps take chunks of tiles
+    int max_blocks = 0;         // most blocks of a mover launch (0: no limit; for tests)
     std::vector<int> collide_nsteps;      // the distinct subcycling factors of colliding species
     double* kin = nullptr;    // k_kinetic's block sums
     char* diag = nullptr;     // the diagnostics' packet of one instance (pic_moments)
@@ -592,6 +593,15 @@ bool full_step(const pic_handle* h, int64_t n)
 // kBorisRounds tiles per resident warp, twice as many) instead of the resident grid, whose
 // warps' tile counts differ by one (1.6 M particles, 3.5 tiles a warp: 78.1 us a step
 // against 80.6, 2 tiles 81.1; 39 M: 1,107 at one, 1,099 at two against 1,136).
+// A batch whose segments are short against the resident grid's stride, so that a warp's next
+// tile would lie in another segment every time (its constants, node arrays and tile range
+// waited for anew), walks the resident grid in chunks as well, sized on the device from the
+// tiles alive (kSpread).  From two segments a stride on: 20 M particles, FP64, 500
+// instances of 100 cells 257 -> 192 us a step, 60 of 5,000 cells 232 -> 208; FP32 142 -> 105
+// and 133 -> 117; at fewer the stride is better (24 uneven instances, 17 M particles, 3,500
+// tiles a segment: 277 us FP64, 142 FP32; in chunks of 8 290 and 154).  With magnetic field
+// (FP32, direct loads) from eight on: 500 of 100 cells 203 -> 191, but 128 uneven ones, 1,400
+// tiles a segment, 250 -> 260.
 constexpr int kMoveChunk = 8;
 constexpr int64_t kBorisRounds = 16;
 // The sort step in the same manner: a block takes kSortChunk consecutive rounds of its
@@ -638,6 +648,7 @@ int launch_move(pic_handle* h, bool move, int phase = kPlain)
         const MoveMode mode = full ? MoveMode::kFull : h->mode;
         const int nt = sort ? h->nt_sort : h->nt;
         int grid = sort ? h->grid_sort : full ? h->grid_full : h->grid_move;
+        if (h->max_blocks > 0) grid = std::min(grid, h->max_blocks);
         const int64_t nw = nt / 32;
         const bool boris64 = !sort && mag && h->precision == PIC_FP64;
         if (sort) {
@@ -646,9 +657,12 @@ int launch_move(pic_handle* h, bool move, int phase = kPlain)
             a.chunk = h->max_tiles >= std::min(h->chunk_rounds, kBorisRounds) * nw * grid ? 2 : 1;
         } else if (h->max_tiles >= h->chunk_rounds * nw * grid) {
             a.chunk = h->precision == PIC_FP64 ? 2 * kMoveChunk : kMoveChunk;
+        } else if ((mag ? 8 : 2) * h->max_tiles < (int64_t)h->nseg * nw * grid) {
+            a.chunk = kSpread;
         }
-        const int64_t blocks = (h->max_tiles + nw * a.chunk - 1) / (nw * a.chunk);
+        const int64_t per = nw * std::max(a.chunk, 1), blocks = (h->max_tiles + per - 1) / per;
         if (a.chunk > 1 || boris64 || blocks < grid) grid = (int)std::max<int64_t>(blocks, 1);
+        if (h->max_blocks > 0) grid = std::min(grid, h->max_blocks);
         h->kernels += 1;
         const cudaError_t e =
             h->precision == PIC_FP64
@@ -1123,6 +1137,7 @@ int pic_create(const pic_config* cfg, pic_handle** out)
     if (const char* v = std::getenv("BITPIC_PAIR_MIN_SLOTS")) h->full_min = std::atoll(v);
     if (const char* v = std::getenv("BITPIC_AHEAD_TILES")) h->ahead_tiles = std::atoll(v);
     if (const char* v = std::getenv("BITPIC_CHUNK_ROUNDS")) h->chunk_rounds = std::atoll(v);
+    if (const char* v = std::getenv("BITPIC_MOVE_BLOCKS")) h->max_blocks = std::atoi(v);
     for (const SegParams& P : h->segh)
         if (P.collide && std::find(h->collide_nsteps.begin(), h->collide_nsteps.end(), P.nstep) ==
                              h->collide_nsteps.end())
