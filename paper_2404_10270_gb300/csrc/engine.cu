@@ -1003,6 +1003,7 @@ int pic_create(const pic_config* cfg, pic_handle** out)
 
     // segment and node layout
     int64_t slot = 0, snode = 0, inode = 0, ev = 0;
+    double candidates = 0.0, events_likely = 0.0;  // a step, of full segments
     for (int i = 0; i < h->ninst; ++i) {
         const pic_instance& I = h->inst[i];
         InstParams ip;
@@ -1103,6 +1104,8 @@ int pic_create(const pic_config* cfg, pic_handle** out)
                 const double wall = I.bc == PIC_BC_PERIODIC ? 0.0 : (I.bc == PIC_BC_SOURCE ? 2.0 : 1.0) / 16.0;
                 const double frac = std::min(1.0, 4.0 * Pc + wall);
                 h->rare_cap += (int64_t)std::ceil((double)P.cap * frac);
+                candidates += (double)P.cap * Pc;
+                events_likely += (double)P.cap * (1.5 * Pc + wall);
             }
             h->segh.push_back(P);
         }
@@ -1169,7 +1172,13 @@ int pic_create(const pic_config* cfg, pic_handle** out)
         return bail(PIC_ECUDA);
     }
     h->sms = prop.multiProcessorCount;
-    h->grid_events = (int)std::min<int64_t>((h->rare_cap - 65536 + 127) / 128, (int64_t)4 * h->sms);
+    // Blocks for the events a step may well have, but one for every expected candidate (k_events
+    // spreads a few over the SMs) on all but a few SMs, where the field phase beside it
+    // finds room for its large blocks (152 blocks: 17.0 against 14.3 us a step for 1,000 cells
+    // in FP32).  (From the queue's capacity, which a small store bounds, a collisional plasma
+    // of 51,200 particles got 32 blocks: FP64, at a candidate in 200 39 against 17 us a step.)
+    h->grid_events = (int)std::min<double>((events_likely + 127.0) / 128.0, 4.0 * h->sms);
+    h->grid_events = std::max(h->grid_events, (int)std::min<double>(candidates, 0.95 * h->sms));
     h->grid_events = std::max(h->grid_events, std::min(h->sms, 32));
     // one warp per requested target cell: at most the ionization events of a step
     h->grid_victims = (int)std::min<int64_t>((std::max<int64_t>(h->ev_total, 1) + 3) / 4, (int64_t)4 * h->sms);
