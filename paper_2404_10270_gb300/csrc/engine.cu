@@ -1222,7 +1222,12 @@ int pic_create(const pic_config* cfg, pic_handle** out)
     if (rc == PIC_OK && h->any_target) rc = dalloc(h, &h->tcount, (size_t)snode);
     if (rc == PIC_OK && h->any_target) rc = dalloc(h, &h->treq, (size_t)snode);
     if (rc == PIC_OK && h->any_target) rc = dalloc(h, &h->vlist, (size_t)std::max<int64_t>(ev, 1));
-    const size_t diag_bytes = sizeof(DiagHead) + (size_t)(PIC_MAX_SPECIES + 2) * h->max_nodes * 8;
+    // (the largest instance's packet: its densities, the potential where there is one, E)
+    size_t diag_bytes = 0;
+    for (const pic_instance& I : h->inst)
+        diag_bytes = std::max(diag_bytes, (size_t)(I.nspecies + (I.field == PIC_FIELD_POISSON) + 1) *
+                                              (size_t)(I.ncells + 1) * 8);
+    diag_bytes += sizeof(DiagHead);
     if (rc == PIC_OK) rc = dalloc(h, &h->diag, diag_bytes);
     h->diag_h_bytes = std::min<size_t>(diag_bytes, kDiagPinned);
     if (rc == PIC_OK && cudaMallocHost((void**)&h->diag_h, h->diag_h_bytes) != cudaSuccess) {
