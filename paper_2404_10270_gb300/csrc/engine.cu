@@ -168,6 +168,7 @@ struct pic_handle {
     // autotuning of the mover block size and the sort interval (see tune_step)
     bool tune_block = false, tune_sort = false;
     int tune_phase = 0;        // 0 idle/done, 1 block sizes, 2 sort intervals
+    bool tune_warm = false;  // a cycle before the first candidate's
     int tune_idx = 0;          // candidate being measured
     double tune_best = 1e300;  // best cost per particle-step so far (ms)
     int tune_best_val = 0;
@@ -857,9 +858,13 @@ int live_total(pic_handle* h, double* out)
 // (deposits are integer, random draws are keyed by particle id, the sort only permutes),
 // so the tuner measures candidates on the first steps of the real run: one sort cycle
 // per candidate, block sizes first (at sort interval 20), then sort intervals.  The
-// choice is cached per GPU and size bucket (precision, magnetised or not, log2 of the
-// particle count and of the mean cell count) in a JSON file: $BITPIC_TUNE_CACHE, else
-// $HOME/.cache/bitpic/autotune.json.
+// choice is cached per GPU, mover generation and size bucket (precision, magnetised or not,
+// subcycled or not, log2 of the particle count and of the mean cell count) in a JSON file:
+// $BITPIC_TUNE_CACHE, else $HOME/.cache/bitpic/autotune.json.  kMoverGeneration goes up with
+// every change of the mover or the sort step that may move the best choice, so that a file
+// from an older build is measured anew (196.6 M particles, FP32: 512 threads were best once,
+// 128 are now).
+constexpr int kMoverGeneration = 2;
 const int kTuneBlocks[] = {128, 256, 512};
 const int kTuneSorts[] = {10, 20, 40, 80};
 std::mutex g_tune_mutex;
@@ -934,8 +939,9 @@ void tune_begin(pic_handle* h)
     const int lp = (int)std::floor(std::log2((double)std::max<int64_t>(np, 1)));
     const int lc = (int)std::floor(std::log2((double)std::max<int64_t>(cells / h->ninst, 1)));
     char key[400];
-    std::snprintf(key, sizeof(key), "%s|%s|%s|p%d|c%d", h->gpu_name,
-                  h->precision == PIC_FP64 ? "fp64" : "fp32", h->any_mag ? "mag" : "nomag", lp, lc);
+    std::snprintf(key, sizeof(key), "%s|m%d|%s|%s|%s|p%d|c%d", h->gpu_name, kMoverGeneration,
+                  h->precision == PIC_FP64 ? "fp64" : "fp32", h->any_mag ? "mag" : "nomag",
+                  h->any_subcycle ? "sub" : "all", lp, lc);
     h->tune_key = key;
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     const auto m = tune_cache_read();
@@ -948,6 +954,7 @@ void tune_begin(pic_handle* h)
         return;
     }
     h->tune_phase = h->tune_block ? 1 : 2;
+    h->tune_warm = true;
     h->tune_idx = 0;
     h->tune_best = 1e300;
     if (h->tune_phase == 1) set_block(h, kTuneBlocks[0]);
@@ -1594,23 +1601,50 @@ int pic_step(pic_handle* h, int64_t nsteps)
         const int64_t K = h->sort_interval;
         // autotuning: time one whole sort cycle per candidate on the real run
         if (h->tune_phase && K > 0 && h->step_h % K == 0 && nsteps - n >= K) {
+            // one cycle first that nobody is charged for: the kernels of a step are loaded on
+            // their first launch (milliseconds)
+            if (h->tune_warm) {
+                for (int64_t k = 0; k < K; ++k)
+                    if ((rc = enqueue_step(h))) return rc;
+                n += K;
+                h->tune_warm = false;
+                continue;
+            }
             // the cost per particle-step: sources and ionization change the particle
             // count from one candidate's cycle to the next
             double live0 = 0.0, live1 = 0.0;
             if ((rc = live_total(h, &live0))) return rc;
             cudaEvent_t ea = take_event(h), eb = take_event(h);
             CUDA_TRY(h, cudaEventRecord(ea, h->stream));
-            for (int64_t k = 0; k < K; ++k)
+            // (a step with the kFull mover, the first after a load and one in 127, would
+            // count against the candidate whose cycle it falls into: timed apart)
+            std::vector<std::pair<cudaEvent_t, cudaEvent_t>> apart;
+            for (int64_t k = 0; k < K; ++k) {
+                const bool full = full_step(h, h->step_h) && (h->step_h + 1) % K != 0;
+                if (full) {
+                    apart.emplace_back(take_event(h), take_event(h));
+                    CUDA_TRY(h, cudaEventRecord(apart.back().first, h->stream));
+                }
                 if ((rc = enqueue_step(h))) return rc;
+                if (full) CUDA_TRY(h, cudaEventRecord(apart.back().second, h->stream));
+            }
             CUDA_TRY(h, cudaEventRecord(eb, h->stream));
             CUDA_TRY(h, cudaEventSynchronize(eb));
             float ms = 0.f;
             CUDA_TRY(h, cudaEventElapsedTime(&ms, ea, eb));
+            for (const auto& e : apart) {
+                float t = 0.f;
+                CUDA_TRY(h, cudaEventElapsedTime(&t, e.first, e.second));
+                ms -= t;
+                h->event_pool.push_back(e.first);
+                h->event_pool.push_back(e.second);
+            }
             h->event_pool.push_back(ea);
             h->event_pool.push_back(eb);
             n += K;
             if ((rc = live_total(h, &live1))) return rc;
-            const double per = ms / ((double)K * std::max(0.5 * (live0 + live1), 1.0));
+            const double steps = (double)std::max<int64_t>(K - (int64_t)apart.size(), 1);
+            const double per = ms / (steps * std::max(0.5 * (live0 + live1), 1.0));
             if (h->tune_phase == 1) {
                 if (per < h->tune_best) { h->tune_best = per; h->tune_best_val = h->nt; }
                 if (++h->tune_idx < 3) {
