@@ -1085,7 +1085,6 @@ k_move(const __grid_constant__ MoveArgs a)
     __shared__ __align__(16) uint32_t s_dwin[NT / 32][DepWin<Q>::words + CrossScratch<T>::words];
     uint32_t* const dwin = s_dwin[threadIdx.x >> 5];
     double* const scr = reinterpret_cast<double*>(dwin + DepWin<Q>::words);
-    dep_win_clear<Q>(dwin);
     // (fewer than 2^31 tiles: 2^38 particles would not fit)
     const int total = (int)a.tile_start[a.nseg];
     // the tile ahead: its segment (tiles only increase) with that segment's last tile + 1 and
@@ -1094,6 +1093,8 @@ k_move(const __grid_constant__ MoveArgs a)
     const int chunk = (MAG && sizeof(T) == 8) || a.chunk != kSpread
                           ? a.chunk : spread_chunk(total, gridDim.x * (NT / 32));
     int tile = (blockIdx.x * (NT / 32) + (threadIdx.x >> 5)) * chunk, left = chunk - 1;
+    if (tile >= total) return;  // (blocks for a reserve that is not alive)
+    dep_win_clear<Q>(dwin);
     int sa = 0, sa_end = -1;
     int64_t ahead0 = 0, ahead_end = 0, ahead = 0;
     const auto next = [&]() {
