@@ -923,18 +923,12 @@ __device__ __forceinline__ int test_clock(const MoveArgs& a, const SegParams& P,
     return (int)(((uint32_t)c & kCellMask) | clk);
 }
 
-// The tests are called, not inlined: inlined, their registers moved the schedule of the
-// loop (196.6 M particles, FP32: mover 650 against 646 us, the sort step 2.28 against
-// 2.22 ms); and with them called the Boris form wants rare_quad called too (39 M particles
-// in FP32: 230 us, inlined 250), the others not (650 against 647).
-//
 // The clock tests of a quad that is in memory again after its step (plain step), `test` a bit
 // per quad position.  Only the clocks are left to do: the quad's move and its share of the
 // warp's deposit are the common path's.  (Doing such quads over one particle at a time, with
 // two 64-bit atomics each, took 5.5 ms for the 14.3 M particles of a 256-cell plasma on the
 // steps on which every clock tests, and 72 us on the others.)
-static __device__ __noinline__ void test_quad(const MoveArgs& a, int s, int64_t step, int64_t slot,
-                                              int test)
+__device__ __forceinline__ void test_quad(const MoveArgs& a, int s, int64_t step, int64_t slot, int test)
 {
     const SegParams& P = a.seg[s];
     int64_t mown;
@@ -948,6 +942,17 @@ static __device__ __noinline__ void test_quad(const MoveArgs& a, int s, int64_t 
             a.cell[slot + k] = test_clock(a, P, s, step, mown, dgrid,
                                           k == 0 ? id.x : k == 1 ? id.y : k == 2 ? id.z : id.w,
                                           k == 0 ? c.x : k == 1 ? c.y : k == 2 ? c.z : c.w, slot + k);
+}
+
+// test_quad called: inlined, its registers moved the schedule of the plain push's loop (196.6 M
+// particles, FP32: 650 against 646 us; the sort step, below, 2.28 against 2.22 ms).  The
+// Boris form takes it inlined, with rare_quad: a call reads the kernel's arguments through
+// memory, which every step with an ionization product waits for (256 cells x 100 x 2: FP32
+// 22.7 against 20.8 us a step, FP64 36.7 against 34.6).
+static __device__ __noinline__ void test_quad_called(const MoveArgs& a, int s, int64_t step,
+                                                     int64_t slot, int test)
+{
+    test_quad(a, s, step, slot, test);
 }
 
 // The same of a quad staged for the sort at the places pk of the chunk's arrays (-1: none);
@@ -1032,14 +1037,6 @@ __device__ __forceinline__ int spread_chunk(int total, int warps)
 {
     const int tiles = max((total + warps - 1) / warps, 1), times = max((tiles + 16) / 32, 1);
     return (tiles + times - 1) / times;
-}
-
-// rare_quad called: the Boris form's loop, whose registers are scarce (see test_quad).
-template <typename T>
-static __device__ __noinline__ void rare_quad_boris(const MoveArgs& a, int s, bool smag, int64_t step,
-                                                    int64_t slot)
-{
-    rare_quad<T, true>(a, s, smag, step, slot);
 }
 
 // The fused time step.  Work unit: a warp tile of 32 quads (128 consecutive particles
@@ -1270,9 +1267,9 @@ k_move(const __grid_constant__ MoveArgs a)
                                      MOVE && SUB && !moves ? nullptr : a.dep + node0,
                                      a.hist_out ? a.hist_out + node0 : nullptr, dwin);
         if (!FULL && todo != 0) {
-            if (todo > 0) test_quad(a, s, step, slot, todo);
-            else if (MAG) rare_quad_boris<T>(a, s, smag, step, slot);
-            else rare_quad<T, MAG>(a, s, smag, step, slot);
+            if (todo < 0) rare_quad<T, MAG>(a, s, smag, step, slot);
+            else if (MAG) test_quad(a, s, step, slot, todo);
+            else test_quad_called(a, s, step, slot, todo);
         }
     }
 }
