@@ -660,7 +660,8 @@ int launch_move(pic_handle* h, bool move, int phase = kPlain)
             a.chunk = h->max_tiles >= std::min(h->chunk_rounds, kBorisRounds) * nw * grid ? 2 : 1;
         } else if (h->max_tiles >= h->chunk_rounds * nw * grid) {
             a.chunk = h->precision == PIC_FP64 ? 2 * kMoveChunk : kMoveChunk;
-        } else if ((mag ? 8 : 2) * h->max_tiles < (int64_t)h->nseg * nw * grid) {
+        } else if (can_spread(h->precision == PIC_FP64, mag, nt) &&
+                   (mag ? 8 : 2) * h->max_tiles < (int64_t)h->nseg * nw * grid) {
             a.chunk = kSpread;
         }
         const int64_t per = nw * std::max(a.chunk, 1), blocks = (h->max_tiles + per - 1) / per;

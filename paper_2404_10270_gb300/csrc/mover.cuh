@@ -1033,6 +1033,13 @@ __device__ __forceinline__ void rare_quad(const MoveArgs& a, int s, bool smag, i
 // kSpread): up to some 32 (8: 209 against 203 us for 500 instances of 100 cells, FP64), so
 // many that all warps get the same number of chunks, from the tiles that are alive.
 constexpr int kSpread = 0;
+// Not the FP64 Boris form, which is launched a block for every NT/32 or twice as many tiles, nor
+// FP64 in blocks of 512 threads, whose 64 registers have none to spare for it (196.6 M
+// particles: 1.460 against 1.466 ms; as little for quad_walls).
+__host__ __device__ constexpr bool can_spread(bool f64, bool mag, int nt)
+{
+    return !(f64 && (mag || nt == 512));
+}
 __device__ __forceinline__ int spread_chunk(int total, int warps)
 {
     const int tiles = max((total + warps - 1) / warps, 1), times = max((tiles + 16) / 32, 1);
@@ -1069,6 +1076,7 @@ k_move(const __grid_constant__ MoveArgs a)
     using Q = typename Prec<T>::Q;
     using T2 = typename Prec<T>::T2;
     constexpr bool PF = MODE == MoveMode::kAhead, FULL = MODE == MoveMode::kFull;
+    constexpr bool WALLS = !MAG && !(sizeof(T) == 8 && NT == 512);
     static_assert(!(PF && MAG), "the Boris form loads directly");
     const int lane = threadIdx.x & 31;
     T* const offp = static_cast<T*>(a.off);
@@ -1086,8 +1094,7 @@ k_move(const __grid_constant__ MoveArgs a)
     const int total = (int)a.tile_start[a.nseg];
     // the tile ahead: its segment (tiles only increase) with that segment's last tile + 1 and
     // slots (ahead0: as if tile 0 were its), and the slot of the lane's quad
-    // (the FP64 Boris form is launched a block for every NT/32 or twice as many tiles)
-    const int chunk = (MAG && sizeof(T) == 8) || a.chunk != kSpread
+    const int chunk = !can_spread(sizeof(T) == 8, MAG, NT) || a.chunk != kSpread
                           ? a.chunk : spread_chunk(total, gridDim.x * (NT / 32));
     int tile = (blockIdx.x * (NT / 32) + (threadIdx.x >> 5)) * chunk, left = chunk - 1;
     if (tile >= total) return;  // (blocks for a reserve that is not alive)
@@ -1222,8 +1229,8 @@ k_move(const __grid_constant__ MoveArgs a)
             } else {
                 bool due;
                 int walls = 0;
-                const bool rare = quad_fast<T, MAG, !MAG>(P, F, smag, static_cast<const T2*>(a.accel) + node0,
-                                                          c, f, ux, uy, uz, moved, due, walls, scr);
+                const bool rare = quad_fast<T, MAG, WALLS>(P, F, smag, static_cast<const T2*>(a.accel) + node0,
+                                                           c, f, ux, uy, uz, moved, due, walls, scr);
                 if (rare && act) todo = -1;
                 if (due && act && !rare) {
                     const int ev = quad_due(F, c);
@@ -1232,7 +1239,7 @@ k_move(const __grid_constant__ MoveArgs a)
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         if (ev >> k & 1) queue_rare(a, s, slot + k, kRareCandidate);
-                        if (!MAG && (walls >> k & 17))
+                        if (WALLS && (walls >> k & 17))
                             queue_rare(a, s, slot + k, walls >> k & 1 ? kRareWallLow : kRareWallHigh);
                     }
                 }
