@@ -158,9 +158,9 @@ struct pic_handle {
     int grid_sort = 0;
     int grid_full = 0;  // grid of the mover's kFull variant
     // threads per block of the step that ends a sort cycle, apart from the other steps': its
-    // four block-wide barriers a round cost less in small blocks (196.6 M particles: 2.18 /
-    // 2.27 ms at 128 / 256 threads in FP32, 3.83 / 4.14 in FP64); `$BITPIC_SORT_BLOCK` (128,
-    // 256 or 512) overrides it
+    // four block-wide barriers a round cost less in small blocks (196.6 M particles: 2.17 /
+    // 2.35 / 2.70 ms at 128 / 256 / 512 threads in FP32, 3.57 / 4.10 / 5.80 in FP64);
+    // `$BITPIC_SORT_BLOCK` (128, 256 or 512) overrides it
     int nt_sort = 128;
     int state = PIC_OK;
     std::string last_error;
@@ -590,8 +590,9 @@ bool full_step(const pic_handle* h, int64_t n)
 // particles, FP32, 256-thread blocks: 0.644 ms against 0.692 (16 tiles 0.646, 32 0.664);
 // FP64 1.41 (16 tiles; 8: 1.43) against 1.47; 128 magnetized instances, FP32: 0.938 against
 // 1.060.  Below chunk_rounds tiles per resident warp the resident grid wins, whose warps
-// are set up once (98 M particles, 158 tiles a warp: 389 against 392 us a step; 49 M: 199
-// against 207; 30 M: 131 against 133).  The FP64 Boris form, which the FP64 pipe bounds,
+// are set up once (FP32 in 256-thread blocks, tiles a warp: 96 206 against 209 us a step, 158 326
+// against 325, 183 378 against 377, 207 427 against 446, 241 496 against 510; FP64 at 211 703
+// against 735, at 128 442 against 446).  The FP64 Boris form, which the FP64 pipe bounds,
 // wants its tiles spread evenly over the SMs: a block for every NT/32 tiles (from
 // kBorisRounds tiles per resident warp, twice as many) instead of the resident grid, whose
 // warps' tile counts differ by one (1.6 M particles, 3.5 tiles a warp: 78.1 us a step
@@ -603,13 +604,15 @@ bool full_step(const pic_handle* h, int64_t n)
 // instances of 100 cells 257 -> 192 us a step, 60 of 5,000 cells 232 -> 208; FP32 142 -> 105
 // and 133 -> 117; at fewer the stride is better (24 uneven instances, 17 M particles, 3,500
 // tiles a segment: 277 us FP64, 142 FP32; in chunks of 8 290 and 154).  With magnetic field
-// (FP32, direct loads) from eight on: 500 of 100 cells 203 -> 191, but 128 uneven ones, 1,400
-// tiles a segment, 250 -> 260.
+// (FP32, direct loads of five arrays) only below 64 tiles a segment: 2,000 of 50 cells,
+// 36 tiles, 232 -> 204, but 512 uneven ones of 573 tiles, 50 M particles, 496 -> 541, of 115
+// 193 -> 196.
 constexpr int kMoveChunk = 8;
 constexpr int64_t kBorisRounds = 16;
 // The sort step in the same manner: a block takes kSortChunk consecutive rounds of its
-// NT/32 tiles and ends.  196.6 M particles: FP32 2.30 -> 2.18 ms (8 rounds 2.21), FP64 4.01 ->
-// 3.83; 49 M FP32 559 -> 550 us (8: 568).  From kSortRounds tiles per resident warp.
+// NT/32 tiles and ends.  196.6 M particles, before its registers were its own: FP32 2.30 -> 2.18
+// ms (8 rounds 2.21), FP64 4.01 -> 3.83; 49 M FP32 559 -> 550 us (8: 568).  From kSortRounds
+// tiles per resident warp.
 constexpr int kSortChunk = 4;
 constexpr int64_t kSortRounds = 32;
 
@@ -661,7 +664,8 @@ int launch_move(pic_handle* h, bool move, int phase = kPlain)
         } else if (h->max_tiles >= h->chunk_rounds * nw * grid) {
             a.chunk = h->precision == PIC_FP64 ? 2 * kMoveChunk : kMoveChunk;
         } else if (can_spread(h->precision == PIC_FP64, mag, nt) &&
-                   (mag ? 8 : 2) * h->max_tiles < (int64_t)h->nseg * nw * grid) {
+                   (mag ? h->max_tiles < 64 * (int64_t)h->nseg
+                        : 2 * h->max_tiles < (int64_t)h->nseg * nw * grid)) {
             a.chunk = kSpread;
         }
         const int64_t per = nw * std::max(a.chunk, 1), blocks = (h->max_tiles + per - 1) / per;
