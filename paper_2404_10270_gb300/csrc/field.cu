@@ -119,8 +119,9 @@ __device__ __forceinline__ i128 smoothed_charge(const FieldArgs& f, const InstPa
 // Snapshot each segment's slot count, rounded up to a whole quad, as the count the next step
 // moves, and build its tile list (TileArgs); one block, kTileBatch segments of a thread in
 // flight at a time (one after another, 63 a thread in blocks of 32, they took 62 us of the
-// field phase of 1,000 31-cell instances).
-constexpr int kTileBatch = 8;
+// field phase of 1,000 31-cell instances, 14 now; eight cost the field kernels 16 registers:
+// 512 uneven instances, 1.0 M nodes, 73 -> 80 us).
+constexpr int kTileBatch = 4;
 __device__ __forceinline__ void build_tiles(const SegParams* seg, const TileArgs& t, i128* sh)
 {
     const int nseg = t.nseg;
