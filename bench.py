@@ -52,8 +52,9 @@ FP64_OPS_PER_PARTICLE_BORIS = 12
 FP64_PEAK_INSTR_PER_S = 2 * 152 * 2.07e9
 # Mover threads per block of the 196.6 M-particle workload in both forms (the step that
 # ends a sort cycle has its own block size, 128): with warps that take chunks of tiles, small
-# blocks follow the store most closely (0.748 / 0.764 / 0.770 ms per step at 128 / 256 / 512 in
-# FP32, 1.52 / 1.56 / 1.61 in FP64).  The subcycled variant and the paper's test case keep 256.
+# blocks follow the store most closely (0.761 / 0.764 / 0.779 ms per step at 128 / 256 / 512 in
+# FP32 over a sort cycle, 1.52 / 1.55 / 1.63 in FP64).  The subcycled variant and the paper's
+# test case keep 256.
 LARGE_BLOCK = 128
 
 
